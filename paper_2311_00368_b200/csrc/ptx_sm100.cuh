@@ -140,6 +140,23 @@ __device__ __forceinline__ void wait_for_primary_grid()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// ---- one thread of a warp ---------------------------------------------------------------------------
+// True in one thread of a converged warp, always the same one (all 32 lanes must call it).  Inside `if (elect_one())` the
+// compiler knows that a single thread is active, so the operands of tcgen05.mma and of bulk copies, which the hardware
+// takes from uniform registers, are moved there once; inside `if (lane == 0)` it serialises every such instruction over
+// the threads that might be active.  Measured on the issue loop of twelve 128 x 128 x 8 tf32 MMAs (64 cycles each on
+// the tensor pipe) behind one barrier check: 67 cycles per MMA elected, 77 with lane 0 (196 against 290 with one MMA per loop).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // ---- fences ---------------------------------------------------------------------------------------
 // Makes this thread's generic-proxy shared-memory writes visible to the async proxy (TMA, tcgen05).
 __device__ __forceinline__ void fence_proxy_async_smem()

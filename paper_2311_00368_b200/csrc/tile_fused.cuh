@@ -414,7 +414,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         // for the tensor core again as soon as its last columns have been read.
         const uint32_t stage = flush_stage + (uint32_t)q * 4096;
         if (a.out_tma) {
-            if (lane == 0) ptx::bulk_wait<0>();   // the previous flush's reductions are complete (order of the sums)
+            if (ptx::elect_one()) ptx::bulk_wait<0>();   // the previous flush's reductions are complete (order of the sums)
             __syncwarp();
             // one K split: the output itself, problem = third coordinate; several: the slabs, stacked
             const int y = (a.KS == 1 ? 0 : (prob * a.KS + ks) * a.slab_rows) + m0 + q * 32;
@@ -423,7 +423,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             for (int c = 0; c < a.NT / 16; ++c) {
                 const uint32_t buf = stage + (uint32_t)(c & 1) * 2048;
                 if (c >= 2) {
-                    if (lane == 0) ptx::bulk_wait_read<1>();   // the buffer's previous contents have been read
+                    if (ptx::elect_one()) ptx::bulk_wait_read<1>();   // the buffer's previous contents have been read
                     __syncwarp();
                 }
                 uint32_t r[16];
@@ -447,7 +447,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                                  "r"(r[4 * j]), "r"(r[4 * j + 1]), "r"(r[4 * j + 2]), "r"(r[4 * j + 3]) : "memory");
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     if (first_sum) ptx::tma_store_3d(&tm_out, buf, n0 + c * 16, y, z);
                     else ptx::tma_reduce_add_3d(&tm_out, buf, n0 + c * 16, y, z);
                     ptx::bulk_commit();
@@ -504,7 +504,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
 
     if (warp == kFusedTmaWarp) {
         // ---------------- TMA producer: per block NCH_B chunks of B rows, then NCH_D chunks of D rows ----------------
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             if (!SPMM) { ptx::tma_prefetch_desc(&tm_bhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_blo); }
             if (FUSED) { ptx::tma_prefetch_desc(&tm_dhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_dlo); }
             // Chunk order = the order the MMA thread consumes them: B(0); then per block b:
@@ -553,7 +553,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t idesc1 = ptx::idesc_tf32(kFusedRows, kFusedBlk, false, false);
             const uint32_t idesc2 = a.NT == 64 ? ptx::idesc_tf32(kFusedRows, 64, false, true) : ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
             constexpr uint32_t idesc2_cat = ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
@@ -563,6 +563,16 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             // of three; the flush adds the two halves.
             const bool cat = !EXACT && a.NT == 64;
             int c = 0, ppu = 0;   // chunk counter, P' buffer uses so far
+            // The chunk after the one whose MMAs are being issued is asked for halfway through them: the tensor pipe has
+            // about three MMAs queued then, which hide one barrier check (~100 cycles) but not two in a row.  (Not with
+            // bfloat16 operands: a chunk is a third of the MMAs there, and asking early meant waiting for data: +4%.)
+            const int nchunk = nblk * (NCH_B + Cfg::NCH_D);
+            int arrived = 0;   // chunks known to be in shared memory
+            auto chunk_arrived = [&](int want) -> bool {
+                if (want < arrived || want >= nchunk) return true;
+                arrived = want + 1;
+                return ptx::mbar_wait(full(want % RING), (want / RING) & 1);
+            };
             // balanced partition: the next segment whose A tile GEMM1 will need, and its first block
             int a_seg = 1, a_next = (bal && !SPMM && (int)ptx::lds32(segtab - 8) > 1) ? (int)ptx::lds32(segtab + 32 + kSegStart) : -1;
             auto gemm1 = [&](int b) -> bool {   // P = A_tile * B_block^T over NCH_B chunks
@@ -579,7 +589,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 const uint32_t pacc = tmem + Cfg::COL_P + pb * kFusedBlk;
                 for (int i = 0; i < NCH_B; ++i, ++c) {
                     const int s = c % RING;
-                    if (!ptx::mbar_wait(full(s), (c / RING) & 1)) return false;
+                    if (!chunk_arrived(c)) return false;
                     ptx::tc_fence_after_sync();
                     const uint32_t b_hi = ring + s * kFusedChunk, b_lo = b_hi + kFusedChunk / 2;
 #pragma unroll
@@ -587,6 +597,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                         const uint64_t dbh = ptx::smem_desc(b_hi + k8 * 32, 16, 1024, ptx::kLayoutSw128);
                         const uint64_t dbl = ptx::smem_desc(b_lo + k8 * 32, 16, 1024, ptx::kLayoutSw128);
                         const uint32_t acol = i * 32 + k8 * 8;
+                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
                         ptx::mma_tf32_ts(pacc, tmem + Cfg::COL_AHI + acol, dbh, idesc1, (i | k8) != 0);
                         if (EXACT) continue;   // A and B exact in tf32: no lo terms
                         ptx::mma_tf32_ts(pacc, tmem + Cfg::COL_AHI + acol, dbl, idesc1, 1);
@@ -605,7 +616,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             auto gemm2 = [&](int b, int w) -> bool {   // O += P'_window * D_window
                 const int s = c % RING, ppb = ppu & 1;
                 if (!ptx::mbar_wait(pp_full(ppb), (ppu >> 1) & 1)) return false;
-                if (!ptx::mbar_wait(full(s), (c / RING) & 1)) return false;
+                if (!chunk_arrived(c)) return false;
                 ptx::tc_fence_after_sync();
                 const uint32_t d_hi = ring + s * kFusedChunk, d_lo = d_hi + kFusedChunk / 2;
                 const uint32_t pph = tmem + Cfg::COL_PP + ppb * 64, ppl = pph + 32;
@@ -618,6 +629,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
 #pragma unroll
                     for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
                         const uint64_t ddh = ptx::smem_desc(d_hi + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
+                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
                         ptx::mma_tf32_ts(oacc, pph + k8 * 8, ddh, idesc2_cat, k8 == 0 ? first : 1u);
                         ptx::mma_tf32_ts(oacc, ppl + k8 * 8, ddh, idesc2, 1);
                     }
@@ -625,6 +637,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
 #pragma unroll
                     for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
                         const uint64_t ddh = ptx::smem_desc(d_hi + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
+                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
                         const uint64_t ddl = ptx::smem_desc(d_lo + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
                         ptx::mma_tf32_ts(oacc, pph + k8 * 8, ddh, idesc2, k8 == 0 ? first : 1u);
                         ptx::mma_tf32_ts(oacc, ppl + k8 * 8, ddh, idesc2, 1);
@@ -890,7 +903,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         }
     }
     if (failed) atomicExch(a.status, 1);
-    if (FUSED && (Cfg::DEDICATED_FLUSH ? warp >= Cfg::FLUSH_WARP0 : Cfg::PSETS == 2 ? warp >= 16 : (warp >= 2 && warp < 6)) && lane == 0) {   // this warp's TMA stores / reductions have been performed
+    if (FUSED && (Cfg::DEDICATED_FLUSH ? warp >= Cfg::FLUSH_WARP0 : Cfg::PSETS == 2 ? warp >= 16 : (warp >= 2 && warp < 6)) && ptx::elect_one()) {   // this warp's TMA stores / reductions have been performed
         ptx::bulk_wait<0>();
         ptx::fence_proxy_async_all();
     }
