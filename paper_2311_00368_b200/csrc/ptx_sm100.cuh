@@ -59,6 +59,12 @@ __device__ __forceinline__ uint32_t lds32_off(uint32_t addr)
     return v;
 }
 
+// ORs `m` into a word of shared memory.
+__device__ __forceinline__ void red_or_shared(uint32_t addr, unsigned m)
+{
+    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(m) : "memory");
+}
+
 // Four fp32 additions to global memory in one reduction (no return value); 16-byte aligned address.
 __device__ __forceinline__ void red_add_v4(float *addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {

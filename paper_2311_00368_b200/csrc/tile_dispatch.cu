@@ -184,10 +184,23 @@ b2sp_status pattern_pass(bool prepared, int M, int K, long long nnz, const int *
     if (cudaMemsetAsync(ws, 0, kWsHeaderBytes, st) != cudaSuccess) return B2SP_ERR_CUDA;
     int2 *win = reinterpret_cast<int2 *>(ws + pattern_table_offset(M));
     if (Wk > kMasksMaxWk) return B2SP_ERR_UNSUPPORTED;
-    if (!allow_dynamic_smem<-1>(reinterpret_cast<const void *>(tile_masks_kernel), kMasksMaxWk * 4)) return B2SP_ERR_CUDA;
-    const long long cap = kSMs * 64, rows_all = (long long)M * batch.count;
-    tile_masks_kernel<<<(unsigned)(rows_all < cap ? rows_all : cap), kMasksWarps * 32, (size_t)Wk * 4, st>>>(
-        M, K, Wk, nnz, row_ptr, col_idx, win, flags, sig, sig_dev);
+    const long long rows_all = (long long)M * batch.count;
+    const size_t row_bytes = sizeof(unsigned) * (size_t)masks_row_words(Wk);
+    // A warp per row wins from about 2000 rows on (2048 x 2048 at 20%: 7.8 against 8.4 us; 1024 x 8192 at 30%: 16.5 against
+    // 10.4; 32768 x 8192 at 20%: 62 against 85) unless the rows are long (average 2457 entries on 8192 x 8192: 35.4 against
+    // 31.2 us, 6553 on 4096 x 65536: 71 against 43; 1638 on 32768 x 8192: see above).
+    const bool shared = row_bytes * kMasksRows > kMasksMaxSmem || rows_all < 2000 || nnz / M > 2048;
+    auto launch = [&](auto kernel, long long blocks, int threads, size_t smem) {
+        const long long cap = 1ll << 24;
+        kernel<<<(unsigned)(blocks < cap ? blocks : cap), threads, smem, st>>>(M, K, Wk, nnz, row_ptr, col_idx, win, flags, sig, sig_dev);
+    };
+    if (shared) {
+        if (!allow_dynamic_smem<-1>(reinterpret_cast<const void *>(tile_masks_kernel<true>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
+        launch(tile_masks_kernel<true>, rows_all, kMasksSharedWarps * 32, row_bytes);
+    } else {
+        if (!allow_dynamic_smem<-2>(reinterpret_cast<const void *>(tile_masks_kernel<false>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
+        launch(tile_masks_kernel<false>, (rows_all + kMasksRows - 1) / kMasksRows, kMasksRows * 32, row_bytes * kMasksRows);
+    }
     *launches += 1;
     return cudaGetLastError() == cudaSuccess ? B2SP_OK : B2SP_ERR_CUDA;
 }

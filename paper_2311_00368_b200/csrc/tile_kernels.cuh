@@ -38,117 +38,197 @@ constexpr int kPatternMagic = 0x62327370;
 // ---- window table -------------------------------------------------------------------------------
 // T[r*Wk + w] = (first CSR position of row r whose column is >= 32w, occupancy bit mask of the column
 // window [32w, 32w+32): bit b set <=> column 32w+b is stored).
-// One block of four warps per row (rows differ a lot in length; blocks are scheduled as they finish),
-// one mask word per window of the row in shared memory.  First sweep: the warps read the row's column
-// indices 128 at a time (coalesced, four per lane); a lane merges the bits of its entries that fall
-// into the same window and ORs them into the window's word (shared-memory atomics).  Second sweep: thread = window; the
-// position of a window is the row start plus the entries of all earlier windows (a block prefix sum
-// over the pop counts).  Every window of every row is written, so the table needs no clearing.
+// A row has one mask word per window in shared memory.  First sweep: lane l of a warp reads eight consecutive
+// entries (two 16-byte loads, the next eight in flight meanwhile) and ORs each entry's bit into its window's word.
+// Second sweep: a lane takes two windows; the position of a window is the row start plus the entries of all earlier
+// windows (a prefix sum over the pop counts).  Every window of every row is written, so the table needs no clearing.
 // The table is only meaningful when the columns of each row are strictly increasing and in range;
 // the first sweep checks exactly that and sets flags[kFlagUnsorted] if not.
-constexpr int kMasksWarps = 4;
-constexpr int kMasksMaxWk = 24 * 1024;   // the mask row must fit in the shared memory a block may ask for (96 KB)
+constexpr int kMasksRun = 8;                          // consecutive entries of a lane
+constexpr int kMasksChunk = 32 * kMasksRun;           // entries of a warp's iteration
+constexpr int kMasksMaxWk = 24 * 1024;                // the mask row must fit in the shared memory a block may ask for (96 KB)
+constexpr int kMasksMaxSmem = kMasksMaxWk * 4;
+constexpr int kMasksRows = 8;                         // rows (= warps) of a tile_masks_kernel<false> block
+constexpr int kMasksOwn = 2048;                       // entries of its row that a warp of such a block reads by itself
+constexpr int kMasksSharedWarps = 4;                  // warps of a tile_masks_kernel<true> block
+__host__ __device__ constexpr int masks_row_words(int Wk) { return (Wk + 127) & ~127; }   // (cleared sixteen bytes per lane)
+
+// Entries p .. p + 7 of a row [beg, end): sixteen-byte loads where all of them are inside the array (p is chosen so that
+// their addresses are aligned), single ones of the row otherwise.
+__device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, int nnz, int beg, int end, int p, int (&v)[kMasksRun])
+{
+    if (p >= end) return;
+    if (p >= 0 && p <= nnz - kMasksRun) {
+#pragma unroll
+        for (int i = 0; i < kMasksRun; i += 4) {
+            const int4 x = __ldg(reinterpret_cast<const int4 *>(col_idx + p + i));
+            v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kMasksRun; ++i)
+            if (p + i >= beg && p + i < end) v[i] = __ldg(col_idx + p + i);
+    }
+}
+
+// ORs the bits of a lane's run c (entries p .. p + 7) into the row's words (shared-memory address `words`).  `prev` = the
+// entry before the run, `interior` (the same for the whole warp): every lane's run is inside the row.  false: the row is not
+// strictly increasing or out of range (a table with such a row is not used).  Neighbouring lanes are eight entries apart,
+// so that they hardly ever OR into the same word at the same time (consecutive entries mostly share one).
+__device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev, int p, int beg, int end, int K, uint32_t words, bool interior)
+{
+    auto or_bit = [&](int col) { ptx::red_or_shared(words + 4 * (col >> 5), __funnelshift_l(0u, 1u, col)); };   // 1 << (column within the window)
+    if (interior) {
+        bool ok = (p <= beg || c[0] > prev) && c[0] >= 0 && c[kMasksRun - 1] < K;   // (in order, so the others are in range too)
+#pragma unroll
+        for (int i = 1; i < kMasksRun; ++i) ok = ok && c[i] > c[i - 1];
+        if (!ok) return false;
+#pragma unroll
+        for (int i = 0; i < kMasksRun; ++i) or_bit(c[i]);
+        return true;
+    }
+    const int at = p - beg, len = end - beg;   // an end of the row: entries at .. at + 7 of it, some of them not in it
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < kMasksRun; ++i) {
+        if ((unsigned)(at + i) >= (unsigned)len) continue;
+        const bool in_range = (unsigned)c[i] < (unsigned)K;
+        bad |= !in_range || (at + i > 0 && c[i] <= (i == 0 ? prev : c[i == 0 ? 0 : i - 1]));
+        if (in_range) or_bit(c[i]);
+    }
+    return !bad;
+}
 
 // A batch of `sig.batch` patterns of the same M and K (row_ptr arrays `sig.rp_stride` elements apart, each
 // starting at 0; col_idx arrays `sig.nz_stride` elements apart) gives one table per pattern, stacked:
 // T[(b*M + r)*Wk + w], positions relative to the pattern's own col_idx array.
-__global__ void __launch_bounds__(kMasksWarps * 32)
+//
+// SHARED = false: a block of eight warps has eight rows, a warp to each, so that no row waits for a block-wide barrier
+// between its steps.  A warp reads the first kMasksOwn entries of its row by itself; what is left of longer rows is dealt to
+// all eight warps, so that a long row is not one warp's chain of iterations.  SHARED = true: the four warps of a block
+// share one row throughout, for few rows (which would leave the GPU idle otherwise), for long ones and for rows whose words
+// fill the shared memory.
+// What bounds it: instruction issue (82% of the slots at 32768 rows of 820 entries, 2.7 TB/s; about 30 instructions per
+// 32 entries, the row's fixed part included).  Measured, against a block of four warps per row with two barriers and
+// branches per entry (one 16-byte load per lane and step): 32768 x 8192 at 20% 88 -> 62 us, eight patterns of 4096 x 4096
+// at 20% 61 -> 41 us (those do not begin on 16-byte boundaries), 16384 x 512 at 20% 18 -> 13.5 us, power-law 8192 x 8192 at
+// 30% (SHARED) 38.6 -> 31 us.
+template <bool SHARED>
+__global__ void __launch_bounds__(SHARED ? kMasksSharedWarps * 32 : kMasksRows * 32, SHARED ? 8 : 48 / kMasksRows)
 tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ row_ptr0,
                   const int *__restrict__ col_idx0, int2 *__restrict__ T, int *__restrict__ flags,
                   PatternSignature sig, PatternSignature *__restrict__ sig_out)
 {
-    extern __shared__ __align__(16) unsigned mask[];     // Wk words
+    extern __shared__ __align__(16) unsigned mask_rows[];
     // (inside a stateless tile op the operand-split kernel is launched as a programmatic dependent of this
     // one: the two touch different data and may overlap; that kernel waits for this grid before it ends)
     ptx::launch_dependents();
     if (blockIdx.x == 0 && threadIdx.x == 0) *sig_out = sig;   // what the table is built from
-    __shared__ int warp_total[kMasksWarps];
     constexpr unsigned kFull = 0xffffffffu;
-    constexpr int NT = kMasksWarps * 32;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    constexpr int WARPS = SHARED ? kMasksSharedWarps : 1;       // warps of a row
+    constexpr int ROWS = SHARED ? 1 : kMasksRows;               // rows of the block at a time
+    __shared__ int warp_total[WARPS];
+    __shared__ int4 rest[ROWS];                                 // of each row: problem, first entry, first entry not read yet, end
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int words = masks_row_words(Wk);
+    unsigned *mask = mask_rows + (SHARED ? 0 : warp * words);
+    const uint32_t mask_smem = ptx::smem_u32(mask);
     bool bad = false;
     const long long rows_all = (long long)M * sig.batch;
-    for (long long rowg = blockIdx.x; rowg < rows_all; rowg += gridDim.x) {
-        const int pb = sig.batch == 1 ? 0 : (int)(rowg / M), row = (int)(rowg - (long long)pb * M);   // (no 64-bit division for a single pattern)
+    for (long long row0 = (long long)blockIdx.x * ROWS; row0 < rows_all; row0 += (long long)gridDim.x * ROWS) {
+        const long long rowg = row0 + (SHARED ? 0 : warp);
+        const bool live = SHARED || rowg < rows_all;
+        // (no 64-bit division, which is a library call, where it can be avoided)
+        const int pb = sig.batch == 1 || !live ? 0 : rows_all < 0x7fffffffll ? (int)((unsigned)rowg / (unsigned)M) : (int)(rowg / M);
+        const int row = live ? (int)(rowg - (long long)pb * M) : 0;
         const int *__restrict__ row_ptr = row_ptr0 + pb * sig.rp_stride;
         const int *__restrict__ col_idx = col_idx0 + pb * sig.nz_stride;
-        const bool vec = (reinterpret_cast<uintptr_t>(col_idx) & 15) == 0;
-        for (int w = threadIdx.x; w < Wk; w += NT) mask[w] = 0u;
-        __syncthreads();
-        const int beg = __ldg(row_ptr + row), end = __ldg(row_ptr + row + 1);
-        // lane l of a warp takes positions p .. p + 3 (one 16-byte load when the array allows it); the
-        // warp's next load is in flight while this one is checked.
-        auto load4 = [&](int p) {
-            int4 c = make_int4(0, 0, 0, 0);
-            if (p >= end) return c;
-            if (vec && p + 3 < nnz) return __ldg(reinterpret_cast<const int4 *>(col_idx + p));
-            c.x = __ldg(col_idx + p);
-            if (p + 1 < end) c.y = __ldg(col_idx + p + 1);
-            if (p + 2 < end) c.z = __ldg(col_idx + p + 2);
-            if (p + 3 < end) c.w = __ldg(col_idx + p + 3);
-            return c;
-        };
-        const int abeg = beg & ~3;
-        int4 c_next = load4(abeg + 128 * wib + 4 * lane);
-        for (int p0 = abeg + 128 * wib; p0 < end; p0 += 128 * kMasksWarps) {
-            const int p = p0 + 4 * lane;
-            const int4 c = c_next;
-            c_next = load4(p + 128 * kMasksWarps);
-            int prev = __shfl_up_sync(kFull, c.w, 1);
-            if (lane == 0 && p > beg) prev = __ldg(col_idx + p - 1);
-            const bool inside = p >= beg && p + 3 < end;
-            const bool in_range = (unsigned)c.x < (unsigned)K && (unsigned)c.y < (unsigned)K &&
-                                  (unsigned)c.z < (unsigned)K && (unsigned)c.w < (unsigned)K;
-            if (inside && in_range) {
-                // common case: four valid entries, almost always in one or two windows
-                bad |= (p > beg && c.x <= prev) || c.y <= c.x || c.z <= c.y || c.w <= c.z;
-                const int wx = c.x >> 5, wy = c.y >> 5, wz = c.z >> 5, ww = c.w >> 5;
-                const unsigned bx = 1u << (c.x & 31), by = 1u << (c.y & 31), bz = 1u << (c.z & 31), bw = 1u << (c.w & 31);
-                atomicOr(&mask[wx], bx | (wy == wx ? by : 0u) | (wz == wx ? bz : 0u) | (ww == wx ? bw : 0u));
-                if (ww != wx) {
-                    atomicOr(&mask[ww], bw | (wz == ww ? bz : 0u) | (wy == ww ? by : 0u));
-                    if (wy != wx && wy != ww) atomicOr(&mask[wy], by);
-                    if (wz != wx && wz != ww) atomicOr(&mask[wz], bz);
-                }
-            } else {
-                auto visit = [&](int q, int col, int before) {
-                    if (q >= beg && q < end) {
-                        const bool ok = (unsigned)col < (unsigned)K;
-                        bad |= !ok || (q > beg && col <= before);
-                        if (ok) atomicOr(&mask[col >> 5], 1u << (col & 31));
-                    }
-                };
-                visit(p, c.x, prev);
-                visit(p + 1, c.y, c.x);
-                visit(p + 2, c.z, c.y);
-                visit(p + 3, c.w, c.z);
-            }
-        }
-        __syncthreads();
-        int run = beg;
-        for (int w0 = 0; w0 < Wk; w0 += NT) {
-            const int w = w0 + threadIdx.x;
-            const unsigned m = w < Wk ? mask[w] : 0u;
-            const int cnt = __popc(m);
-            int incl = cnt;
+        const int beg = live ? __ldg(row_ptr + row) : 0, end = live ? __ldg(row_ptr + row + 1) : 0;
+        int c[kMasksRun], c_next[kMasksRun];
+        // where lane 0 of the row's first run begins: at or up to three entries before the row, so that loads are aligned
+        const int first = beg - ((beg + ((int)(reinterpret_cast<uintptr_t>(col_idx) >> 2) & 3)) & 3);
+        const int own_end = SHARED ? end : (end - first > kMasksOwn ? first + kMasksOwn : end);
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += t;
-            }
-            if (lane == 31) warp_total[wib] = incl;
+        for (int i = 0; i < kMasksRun; ++i) c_next[i] = 0;
+        int p0 = first + (SHARED ? kMasksChunk * warp : 0);
+        if (beg < end) masks_load_run(col_idx, (int)nnz, beg, end, p0 + kMasksRun * lane, c_next);
+        else p0 = own_end;
+        for (int w = (SHARED ? (int)threadIdx.x : lane) * 4; w < words; w += WARPS * 128)
+            *reinterpret_cast<uint4 *>(mask + w) = make_uint4(0u, 0u, 0u, 0u);
+        if (!SHARED && lane == 0) rest[warp] = make_int4(pb, beg, beg < end ? own_end : end, end);
+        if (SHARED) __syncthreads();
+        else __syncwarp();
+        int carry = 0;   // the last entry of the warp's previous iteration
+        for (; p0 < own_end; p0 += kMasksChunk * WARPS) {
+            const int p = p0 + kMasksRun * lane;
+#pragma unroll
+            for (int i = 0; i < kMasksRun; ++i) c[i] = c_next[i];
+            if (p0 + kMasksChunk * WARPS < own_end) masks_load_run(col_idx, (int)nnz, beg, end, p + kMasksChunk * WARPS, c_next);
+            int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
+            if (lane == 0) prev = !SHARED ? carry : p > beg ? __ldg(col_idx + p - 1) : 0;
+            if (!SHARED) carry = __shfl_sync(kFull, c[kMasksRun - 1], 31);
+            bad |= !masks_or_run(c, prev, p, beg, end, K, mask_smem, p0 >= beg && p0 + kMasksChunk <= end);
+        }
+        if (SHARED) {
             __syncthreads();
-            int before = 0, all = 0;
-#pragma unroll
-            for (int i = 0; i < kMasksWarps; ++i) {
-                const int t = warp_total[i];
-                if (i < wib) before += t;
-                all += t;
+        } else if (__syncthreads_or(beg < end && own_end < end)) {
+            // some of the block's rows are longer: their other entries, in chunks dealt to the warps in turn
+            int turn = 0;   // chunks of the rows before
+            for (int r = 0; r < ROWS; ++r) {
+                const int4 q = rest[r];
+                if (q.z >= q.w) continue;
+                const int *__restrict__ ci = col_idx0 + q.x * sig.nz_stride;
+                const int chunks = (q.w - q.z + kMasksChunk - 1) / kMasksChunk;
+                for (int j = (warp - turn) & (ROWS - 1); j < chunks; j += ROWS) {
+                    const int pc = q.z + j * kMasksChunk, p = pc + kMasksRun * lane;
+                    masks_load_run(ci, (int)nnz, q.y, q.w, p, c);
+                    int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
+                    if (lane == 0) prev = __ldg(ci + p - 1);
+                    bad |= !masks_or_run(c, prev, p, q.y, q.w, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
+                }
+                turn += chunks;
             }
-            if (w < Wk) T[(size_t)rowg * Wk + w] = make_int2(run + before + incl - cnt, (int)m);
-            run += all;
-            __syncthreads();   // warp_total and mask are reused
+            __syncthreads();
         }
+        int run = beg;
+        int2 *Trow = T + rowg * Wk;
+        const bool pairs = ((rowg * Wk) & 1) == 0;   // the row's records are 16-byte aligned in twos
+        if (live)
+            for (int w0 = 0; w0 < Wk; w0 += WARPS * 64) {
+                const int w = w0 + 2 * (SHARED ? (int)threadIdx.x : lane);
+                const uint2 m = w < words ? *reinterpret_cast<const uint2 *>(mask + w) : make_uint2(0u, 0u);
+                const int n0 = __popc(m.x), cnt = n0 + __popc(m.y);
+                int incl = cnt;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const int t = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += t;
+                }
+                int before = 0, all;
+                if (!SHARED) {
+                    all = __shfl_sync(kFull, incl, 31);
+                } else {
+                    if (lane == 31) warp_total[warp] = incl;
+                    __syncthreads();
+                    all = 0;
+#pragma unroll
+                    for (int i = 0; i < WARPS; ++i) {
+                        const int t = warp_total[i];
+                        if (i < warp) before += t;
+                        all += t;
+                    }
+                }
+                const int pos = run + before + incl - cnt;
+                if (pairs && w + 1 < Wk) {
+                    *reinterpret_cast<int4 *>(Trow + w) = make_int4(pos, (int)m.x, pos + n0, (int)m.y);
+                } else {
+                    if (w < Wk) Trow[w] = make_int2(pos, (int)m.x);
+                    if (w + 1 < Wk) Trow[w + 1] = make_int2(pos + n0, (int)m.y);
+                }
+                run += all;
+                if (SHARED) __syncthreads();   // warp_total is reused
+            }
+        if (row0 + (long long)gridDim.x * ROWS < rows_all) __syncthreads();   // the words and `rest` are reused
     }
     if (bad) atomicExch(&flags[kFlagUnsorted], 1);
 }

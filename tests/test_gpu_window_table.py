@@ -1,0 +1,112 @@
+"""The window table of a pattern (b2sp_prepare_pattern), entry by entry against numpy, where its kernels branch: rows shorter
+and longer than a warp's own share, few and many rows, column indices that begin on any 4-byte boundary, batches."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+EDGE_LENS = [0, 1, 2, 3, 7, 8, 9, 31, 255, 256, 257, 259, 511, 513, 2046, 2047, 2048, 2049, 2052, 2303, 2305, 2900]
+
+
+@pytest.fixture(scope="module")
+def b():
+    assert torch.cuda.is_available()
+    from paper_2311_00368_b200 import binding
+    return binding
+
+
+def make_rows(rng, lens, K):
+    rp = np.zeros(len(lens) + 1, np.int32)
+    rp[1:] = np.cumsum(lens)
+    ci = np.concatenate([np.sort(rng.choice(K, n, replace=False)) for n in lens]).astype(np.int32)
+    return rp, ci
+
+
+def expected(rp, ci, K):
+    M, Wk = len(rp) - 1, (K + 31) // 32
+    mask = np.zeros((M, Wk), np.uint32)
+    rows = np.repeat(np.arange(M), np.diff(rp))
+    np.bitwise_or.at(mask, (rows, ci >> 5), np.uint32(1) << (ci & 31).astype(np.uint32))
+    count = np.zeros((M, Wk), np.int64)
+    np.add.at(count, (rows, ci >> 5), 1)
+    return mask, rp[:-1, None] + np.cumsum(count, 1) - count
+
+
+def table_of(ws, M, K, batch=1):
+    off = (512 + 4 * M + 255) // 256 * 256
+    off = (off + 1023) // 1024 * 1024
+    Wk = (K + 31) // 32
+    t = ws[off:off + 8 * batch * M * Wk].view(torch.int32).cpu().numpy().reshape(batch, M, Wk, 2)
+    return t[..., 1].view(np.uint32), t[..., 0]
+
+
+def flags_of(ws):
+    return int(ws[320:324].view(torch.int32).item())
+
+
+def device(rp, ci, shift):
+    """The arrays on the GPU, the column indices `shift` elements behind a 16-byte boundary, -1 around them."""
+    buf = torch.full((ci.size + 16,), -1, dtype=torch.int32, device="cuda")
+    view = buf[4 + shift:4 + shift + ci.size]
+    view.copy_(torch.from_numpy(ci))
+    return torch.from_numpy(rp).cuda(), view
+
+
+@pytest.mark.parametrize("M,K,shift", [(44, 2999, 0), (44, 2999, 3), (2200, 2999, 0), (2200, 2999, 1), (2201, 3008, 2), (2500, 4096, 3)])
+def test_table_entries(b, M, K, shift):
+    rng = np.random.default_rng(M + K + shift)
+    # (mostly short rows, so that the average keeps the kernel with a warp per row where M is large)
+    lens = [EDGE_LENS[i % len(EDGE_LENS)] if i % 3 == 0 or M < 100 else int(rng.integers(0, 300)) for i in range(M)]
+    rp, ci = make_rows(rng, lens, K)
+    drp, dci = device(rp, ci, shift)
+    ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
+    b.prepare_pattern(drp, dci, K, ws)
+    mask, pos = table_of(ws, M, K)
+    want_mask, want_pos = expected(rp, ci, K)
+    assert flags_of(ws) == 0
+    assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
+
+
+@pytest.mark.parametrize("M", [44, 2200])
+@pytest.mark.parametrize("row,entry", [(13, 5), (14, 2045), (17, 2048), (20, 2304), (21, 2899), (21, 2050), (9, 255)])
+def test_disorder_is_seen_wherever_it_is(b, M, row, entry):
+    """Two entries of a row swapped, a repeated entry, a column out of range: each raises the flag."""
+    rng = np.random.default_rng(row + entry)
+    K = 2999
+    lens = EDGE_LENS * (M // len(EDGE_LENS)) if M < 100 else EDGE_LENS + [100] * (M - len(EDGE_LENS))
+    rp, ci = make_rows(rng, lens, K)
+    p = int(rp[row]) + min(entry, lens[row] - 1)
+    ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
+    for what in ("swap", "repeat", "below", "above"):
+        bad = ci.copy()
+        if what == "swap":
+            bad[p], bad[p - 1] = ci[p - 1], ci[p]
+        elif what == "repeat":
+            bad[p] = ci[p - 1]
+        else:
+            bad[p] = -1 if what == "below" else K
+        drp, dci = device(rp, bad, 1)
+        b.prepare_pattern(drp, dci, K, ws)
+        assert flags_of(ws) == 1, what
+    drp, dci = device(rp, ci, 1)
+    b.prepare_pattern(drp, dci, K, ws)
+    assert flags_of(ws) == 0
+
+
+@pytest.mark.parametrize("batch,M,K", [(3, 30, 700), (7, 333, 257)])
+def test_batched_tables(b, batch, M, K):
+    rng = np.random.default_rng(batch)
+    probs = [make_rows(rng, [int(rng.integers(0, min(K, 256))) for _ in range(M)], K) for _ in range(batch)]
+    stride = max(ci.size for _, ci in probs) | 1   # odd: most problems begin off a 16-byte boundary
+    ci = np.full((batch, stride), -1, np.int32)
+    for i, (_, c) in enumerate(probs):
+        ci[i, :c.size] = c
+    rp = np.stack([r for r, _ in probs])
+    ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
+    b.prepare_pattern_batched(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), K, ws)
+    mask, pos = table_of(ws, M, K, batch)
+    assert flags_of(ws) == 0
+    for i, (r, c) in enumerate(probs):
+        want_mask, want_pos = expected(r, c, K)
+        assert np.array_equal(mask[i], want_mask) and np.array_equal(pos[i], want_pos)
