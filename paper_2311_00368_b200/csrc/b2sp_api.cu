@@ -2,6 +2,7 @@
 // See include/b2sp.h (and include/b2sp_debug.h) for the contract of every function.
 #include "../../include/b2sp_debug.h"
 
+#include <algorithm>
 #include <climits>
 #include <cstdlib>
 #include <cstdint>
@@ -40,9 +41,13 @@ inline Workspace carve(void *ws)
 thread_local int g_last_algo[3] = {-1, -1, -1};
 thread_local int g_last_launches[3] = {0, 0, 0};
 
-inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
-// alignment a dense operand needs for the four-element loads of the vector kernels (16 bytes of fp32, 8 of bf16)
-template <typename DT> inline bool aligned_vec(const DT *p) { return (reinterpret_cast<uintptr_t>(p) & (4 * sizeof(DT) - 1)) == 0; }
+// The most elements (4, 2 or 1) that may be loaded at a time from a row-major operand of this width: every row begins on such
+// a boundary and has whole groups of them.
+template <typename DT> inline int vec_width(const DT *p, int width, int64_t ld, int64_t batch_stride = 0)
+{
+    const int64_t odd = (int64_t)(reinterpret_cast<uintptr_t>(p) / sizeof(DT)) | width | ld | batch_stride;
+    return (odd & 3) == 0 ? 4 : (odd & 1) == 0 ? 2 : 1;
+}
 template <typename DT> constexpr int dense_dtype() { return sizeof(DT) == 2 ? kDenseBf16 : kDenseF32; }
 
 inline b2sp_status check_launch()
@@ -108,31 +113,48 @@ inline unsigned gated_blocks(unsigned rows, int *gate, unsigned nbatch = 1)
     return gate && rows > cap ? cap : rows;
 }
 
-template <int U, int SPLIT, typename DT>
+template <int V, int U, int SPLIT, typename DT>
 void launch_spmm(dim3 grid, cudaStream_t st, int N, const int *row_ptr, const int *col_idx,
                  const float *values, const DT *D, int64_t ldd, float *O, int64_t ldo,
                  const int *order, int *gate, int *clear)
 {
     const int nrows = (int)grid.x;
     grid.x = gated_blocks(grid.x, gate);
-    launch_row(spmm_row_kernel<U, SPLIT, DT>, grid, 0, st, gate != nullptr || order != nullptr, N, row_ptr, col_idx, values, D, ldd, O, ldo, order,
+    launch_row(spmm_row_kernel<V, U, SPLIT, DT>, grid, 0, st, gate != nullptr || order != nullptr, N, row_ptr, col_idx, values, D, ldd, O, ldo, order,
                gate, nrows, clear);
 }
 
-// Column geometry for a width N on the float4 path: U float4 per lane, SPLIT sub-warps.
+// Column geometry for a width N: U groups of V columns per lane, SPLIT sub-warps.
 struct Geom { int U, SPLIT, slab; };
-inline Geom pick_geom(int N)
+inline Geom pick_geom(int N, int V)
 {
-    if (N <= 32) return {1, 4, 32};
-    if (N <= 64) return {1, 2, 64};
-    if (N <= 128) return {1, 1, 128};
-    if (N <= 256) return {2, 1, 256};
-    return {4, 1, 512};
+    if (V == 4) {
+        if (N <= 32) return {1, 4, 32};
+        if (N <= 64) return {1, 2, 64};
+        if (N <= 128) return {1, 1, 128};
+        if (N <= 256) return {2, 1, 256};
+        return {4, 1, 512};
+    }
+    if (V == 2) {
+        if (N <= 32) return {1, 2, 32};
+        if (N <= 64) return {1, 1, 64};
+        return {2, 1, 128};
+    }
+    if (N <= 16) return {1, 2, 16};
+    if (N <= 32) return {1, 1, 32};
+    if (N <= 64) return {2, 1, 64};
+    return {4, 1, 128};
 }
 
-inline int pick_ku(int Kd) { return Kd <= 64 ? 2 : Kd <= 128 ? 4 : Kd <= 256 ? 8 : 0; }
+// Register groups of A_i per lane (0: A_i in shared memory).
+inline int pick_ku(int Kd, int V)
+{
+    if (Kd <= 64) return 8 / V;
+    if (Kd <= 128) return 16 / V;
+    return V == 4 && Kd <= 256 ? 8 : 0;
+}
 
-template <int KU, typename DT>
+template <int V, int KU, typename DT>
 void launch_sddmm(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const int *col_idx,
                   const float *sv, const DT *A, int64_t lda, const DT *B, int64_t ldb,
                   float *out, const int *order, int *gate, int *clear)
@@ -140,21 +162,21 @@ void launch_sddmm(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const 
     size_t smem = KU == 0 ? sizeof(float) * (size_t)((Kd + 3) & ~3) : 0;
     const int nrows = (int)grid.x;
     grid.x = gated_blocks(grid.x, gate);
-    launch_row(sddmm_row_kernel<KU, DT>, grid, smem, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, sv, A, lda, B, ldb, out, order,
+    launch_row(sddmm_row_kernel<V, KU, DT>, grid, smem, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, sv, A, lda, B, ldb, out, order,
                gate, nrows, clear);
 }
 
-template <int KU, int U, int SPLIT, typename DT>
+template <int V, int KU, int U, int SPLIT, typename DT>
 b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *row_ptr,
                          const int *col_idx, const float *sv, const DT *A, int64_t lda,
                          const DT *B, int64_t ldb, const DT *D, int64_t ldd, float *O,
                          int64_t ldo, const int *order, int *gate, int *clear, const RowBatch &rb)
 {
-    size_t smem = sizeof(float4) * kRowWarps * U * (32 / SPLIT) +
+    size_t smem = sizeof(VecF<V>) * kRowWarps * U * (32 / SPLIT) +
                   (KU == 0 ? sizeof(float) * (size_t)((Kd + 3) & ~3) : 0);
     const bool batched = grid.z > 1;
-    auto kern_b = fusedmm_row_kernel<KU, U, SPLIT, true, DT>;
-    auto kern_1 = fusedmm_row_kernel<KU, U, SPLIT, false, DT>;
+    auto kern_b = fusedmm_row_kernel<V, KU, U, SPLIT, true, DT>;
+    auto kern_1 = fusedmm_row_kernel<V, KU, U, SPLIT, false, DT>;
     if (smem > 48 * 1024) {
         if (smem > 200 * 1024) return B2SP_ERR_UNSUPPORTED;
         if (cudaFuncSetAttribute(batched ? reinterpret_cast<const void *>(kern_b) : reinterpret_cast<const void *>(kern_1),
@@ -172,7 +194,7 @@ b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *r
     return B2SP_OK;
 }
 
-template <int KU, typename DT>
+template <int V, int KU, typename DT>
 b2sp_status dispatch_fused_geom(const Geom &g, dim3 grid, cudaStream_t st, int Kd, int N,
                                 const int *row_ptr, const int *col_idx, const float *sv,
                                 const DT *A, int64_t lda, const DT *B, int64_t ldb,
@@ -180,12 +202,34 @@ b2sp_status dispatch_fused_geom(const Geom &g, dim3 grid, cudaStream_t st, int K
                                 const int *order, int *gate, int *clear, const RowBatch &rb)
 {
 #define B2SP_F(U_, S_) \
-    return launch_fused<KU, U_, S_, DT>(grid, st, Kd, N, row_ptr, col_idx, sv, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
-    if (g.SPLIT == 4) B2SP_F(1, 4);
+    return launch_fused<V, KU, U_, S_, DT>(grid, st, Kd, N, row_ptr, col_idx, sv, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+    if constexpr (V == 4) {
+        if (g.SPLIT == 4) B2SP_F(1, 4);
+    }
     if (g.SPLIT == 2) B2SP_F(1, 2);
     if (g.U == 1) B2SP_F(1, 1);
-    if (g.U == 2) B2SP_F(2, 1);
-    B2SP_F(4, 1);
+    if constexpr (V == 2) B2SP_F(2, 1);
+    else if (g.U == 2) B2SP_F(2, 1);
+    else B2SP_F(4, 1);
+#undef B2SP_F
+}
+
+template <int V, typename DT>
+b2sp_status dispatch_fused_ku(const Geom &g, dim3 grid, cudaStream_t st, int Kd, int N,
+                              const int *row_ptr, const int *col_idx, const float *sv,
+                              const DT *A, int64_t lda, const DT *B, int64_t ldb,
+                              const DT *D, int64_t ldd, float *O, int64_t ldo,
+                              const int *order, int *gate, int *clear, const RowBatch &rb)
+{
+    const int ku = pick_ku(Kd, V);
+#define B2SP_F(KU_) \
+    return dispatch_fused_geom<V, KU_, DT>(g, grid, st, Kd, N, row_ptr, col_idx, sv, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+    if (ku == 8 / V) B2SP_F(8 / V);
+    if (ku == 16 / V) B2SP_F(16 / V);
+    if constexpr (V == 4) {
+        if (ku == 8) B2SP_F(8);
+    }
+    B2SP_F(0);
 #undef B2SP_F
 }
 
@@ -289,20 +333,27 @@ static b2sp_status spmm_rows(int M, int N, const int *row_ptr, const int *col_id
                              const DT *D, long long ldd, float *O, long long ldo, const int *order,
                              int *gate, int *clear, cudaStream_t st)
 {
-    bool vec = N % 4 == 0 && ldd % 4 == 0 && ldo % 4 == 0 && aligned_vec(D) && aligned16(O);
-    if (vec) {
-        Geom g = pick_geom(N);
-        dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab));
-        if (g.SPLIT == 4) launch_spmm<1, 4, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
-        else if (g.SPLIT == 2) launch_spmm<1, 2, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
-        else if (g.U == 1) launch_spmm<1, 1, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
-        else if (g.U == 2) launch_spmm<2, 1, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
-        else launch_spmm<4, 1, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
+    const int V = std::min(vec_width(D, N, ldd), vec_width(O, N, ldo));
+    const Geom g = pick_geom(N, V);
+    dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab));
+#define B2SP_S(V_, U_, S_) launch_spmm<V_, U_, S_, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear)
+    if (V == 4) {
+        if (g.SPLIT == 4) B2SP_S(4, 1, 4);
+        else if (g.SPLIT == 2) B2SP_S(4, 1, 2);
+        else if (g.U == 1) B2SP_S(4, 1, 1);
+        else if (g.U == 2) B2SP_S(4, 2, 1);
+        else B2SP_S(4, 4, 1);
+    } else if (V == 2) {
+        if (g.SPLIT == 2) B2SP_S(2, 1, 2);
+        else if (g.U == 1) B2SP_S(2, 1, 1);
+        else B2SP_S(2, 2, 1);
     } else {
-        dim3 grid(gated_blocks((unsigned)M, gate), (unsigned)((N + 127) / 128));
-        launch_row(spmm_row_scalar_kernel<DT>, grid, 0, st, gate != nullptr || order != nullptr, N, row_ptr, col_idx, values, D, ldd, O, ldo, order,
-                   gate, M, clear);
+        if (g.SPLIT == 2) B2SP_S(1, 1, 2);
+        else if (g.U == 1) B2SP_S(1, 1, 1);
+        else if (g.U == 2) B2SP_S(1, 2, 1);
+        else B2SP_S(1, 4, 1);
     }
+#undef B2SP_S
     return check_launch();
 }
 
@@ -358,6 +409,28 @@ static b2sp_status spmm_impl(int M, int K, int N, long long nnz, const int *row_
     return rc;
 }
 
+// Picks the SDDMM kernel that holds A_i for this Kd.
+template <int V, typename DT>
+static b2sp_status dispatch_sddmm_ku(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const int *col_idx, const float *s_values,
+                                     const DT *A, long long lda, const DT *B, long long ldb, float *out_values, const int *order,
+                                     int *gate, int *clear)
+{
+    const int ku = pick_ku(Kd, V);
+#define B2SP_C(KU_) launch_sddmm<V, KU_, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+    if (ku == 8 / V) { B2SP_C(8 / V); return B2SP_OK; }
+    if (ku == 16 / V) { B2SP_C(16 / V); return B2SP_OK; }
+    if constexpr (V == 4) {
+        if (ku == 8) { B2SP_C(8); return B2SP_OK; }
+    }
+    const size_t smem = sizeof(float) * (size_t)((Kd + 3) & ~3);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(sddmm_row_kernel<V, 0, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return B2SP_ERR_CUDA;
+    B2SP_C(0);
+#undef B2SP_C
+    return B2SP_OK;
+}
+
 // Enqueues the row-family SDDMM.  `gate` != NULL makes it a device-side fallback.
 template <typename DT>
 static b2sp_status sddmm_rows(int M, int Kd, const int *row_ptr, const int *col_idx, const float *s_values,
@@ -365,27 +438,18 @@ static b2sp_status sddmm_rows(int M, int Kd, const int *row_ptr, const int *col_
                               float *out_values, const int *order, int *gate, int *clear, cudaStream_t st)
 {
     dim3 grid((unsigned)M);
-    bool vec = Kd % 4 == 0 && lda % 4 == 0 && ldb % 4 == 0 && aligned_vec(A) && aligned_vec(B) &&
-               Kd <= 40960;
-    if (vec) {
-        switch (pick_ku(Kd)) {
-        case 2: launch_sddmm<2, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear); break;
-        case 4: launch_sddmm<4, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear); break;
-        case 8: launch_sddmm<8, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear); break;
-        default: {
-            size_t smem = sizeof(float) * (size_t)Kd;
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(sddmm_row_kernel<0, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem) != cudaSuccess)
-                return B2SP_ERR_CUDA;
-            launch_sddmm<0, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear);
-        }
-        }
-    } else {
+    if (Kd > kMaxStagedKd) {
         grid.x = gated_blocks(grid.x, gate);
         launch_row(sddmm_row_scalar_kernel<DT>, grid, 0, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb,
                    out_values, order, gate, M, clear);
+        return check_launch();
     }
+    const int V = std::min(vec_width(A, Kd, lda), vec_width(B, Kd, ldb));
+    const b2sp_status rc =
+        V == 4 ? dispatch_sddmm_ku<4, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+        : V == 2 ? dispatch_sddmm_ku<2, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+                 : dispatch_sddmm_ku<1, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear);
+    if (rc != B2SP_OK) return rc;
     return check_launch();
 }
 
@@ -453,24 +517,19 @@ static b2sp_status fused_rows(int M, int Kd, int N, const int *row_ptr, const in
                               int nbatch = 1, const RowBatch &rb = RowBatch{0, 0, 0, 0, 0, 0})
 {
     b2sp_status rc = B2SP_OK;
-    bool vec = N % 4 == 0 && ldd % 4 == 0 && ldo % 4 == 0 && aligned_vec(D) && aligned16(O) &&
-               Kd % 4 == 0 && lda % 4 == 0 && ldb % 4 == 0 && aligned_vec(A) && aligned_vec(B) &&
-               Kd <= 40960 && ((rb.A | rb.B | rb.D | rb.O) & 3) == 0;
-    if (vec) {
-        Geom g = pick_geom(N);
-        dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab), (unsigned)nbatch);
-        switch (pick_ku(Kd)) {
-        case 2: rc = dispatch_fused_geom<2, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb); break;
-        case 4: rc = dispatch_fused_geom<4, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb); break;
-        case 8: rc = dispatch_fused_geom<8, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb); break;
-        default: rc = dispatch_fused_geom<0, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb); break;
-        }
-        if (rc != B2SP_OK) return rc;
-    } else {
+    if (Kd > kMaxStagedKd) {
         dim3 grid(gated_blocks((unsigned)M, gate, (unsigned)nbatch), (unsigned)((N + 127) / 128), (unsigned)nbatch);
         launch_row(fusedmm_row_scalar_kernel<DT>, grid, 0, st, gate != nullptr || order != nullptr, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb,
                    D, ldd, O, ldo, order, gate, M, clear, rb);
+        return check_launch();
     }
+    const int V = std::min({vec_width(A, Kd, lda, rb.A), vec_width(B, Kd, ldb, rb.B), vec_width(D, N, ldd, rb.D), vec_width(O, N, ldo, rb.O)});
+    const Geom g = pick_geom(N, V);
+    dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab), (unsigned)nbatch);
+    rc = V == 4 ? dispatch_fused_ku<4, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+         : V == 2 ? dispatch_fused_ku<2, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+                  : dispatch_fused_ku<1, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb);
+    if (rc != B2SP_OK) return rc;
     return check_launch();
 }
 

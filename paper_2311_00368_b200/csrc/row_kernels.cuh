@@ -24,6 +24,7 @@ constexpr int kRowWarps = 4;
 constexpr int kRowThreads = kRowWarps * 32;
 constexpr int kBuckets = 32;
 constexpr unsigned kFull = 0xffffffffu;
+constexpr int kMaxStagedKd = 40960;   // longest A_i that is staged in shared memory
 
 // ------------------------------------------------------------------------------------------
 // Row binning (work assignment): counting sort of the rows by length bucket
@@ -115,41 +116,66 @@ __device__ __forceinline__ float4 ldg4(const bf16_t *p)   // four consecutive el
     return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
                        __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
 }
+__device__ __forceinline__ float2 ldg2(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+__device__ __forceinline__ float2 ldg2(const bf16_t *p)   // two consecutive elements, 4-byte aligned
+{
+    const unsigned u = __ldg(reinterpret_cast<const unsigned *>(p));
+    return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+}
 __device__ __forceinline__ float ldg1(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ldg1(const bf16_t *p)
 {
     return __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(p)) << 16);
 }
 
-__device__ __forceinline__ void fma4(float4 &acc, float s, const float4 &v)
+
+// V consecutive elements of a dense row, widened to fp32: what a lane loads, multiplies and stores at a time.  V = 4 where
+// every row of every operand begins on a four-element boundary and has whole groups of four, V = 2 where that holds for
+// pairs, V = 1 for any width, leading dimension and address.
+template <int V> struct alignas(4 * V) VecF { float e[V]; };
+template <int V, typename DT>
+__device__ __forceinline__ VecF<V> ldgv(const DT *p)
 {
-    acc.x = fmaf(s, v.x, acc.x);
-    acc.y = fmaf(s, v.y, acc.y);
-    acc.z = fmaf(s, v.z, acc.z);
-    acc.w = fmaf(s, v.w, acc.w);
+    VecF<V> r;
+    if constexpr (V == 4) {
+        const float4 f = ldg4(p);
+        r.e[0] = f.x; r.e[1] = f.y; r.e[2] = f.z; r.e[3] = f.w;
+    } else if constexpr (V == 2) {
+        const float2 f = ldg2(p);
+        r.e[0] = f.x; r.e[1] = f.y;
+    } else {
+        r.e[0] = ldg1(p);
+    }
+    return r;
 }
 
-__device__ __forceinline__ float dot4(const float4 &a, const float4 &b, float acc)
+template <int V>
+__device__ __forceinline__ void fma_v(VecF<V> &acc, float s, const VecF<V> &v)
 {
-    acc = fmaf(a.x, b.x, acc);
-    acc = fmaf(a.y, b.y, acc);
-    acc = fmaf(a.z, b.z, acc);
-    acc = fmaf(a.w, b.w, acc);
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc.e[i] = fmaf(s, v.e[i], acc.e[i]);
+}
+
+template <int V>
+__device__ __forceinline__ float dot_v(const VecF<V> &a, const VecF<V> &b, float acc)
+{
+#pragma unroll
+    for (int i = 0; i < V; ++i) acc = fmaf(a.e[i], b.e[i], acc);
     return acc;
 }
 
 // Geometry of the SPMM sweep.  SPLIT sub-warps of LPN = 32/SPLIT lanes each take alternate
-// entries of a chunk; a lane owns U float4 column groups: columns col0 + (sl + LPN*u)*4.
-template <int U, int SPLIT>
+// entries of a chunk; a lane owns U groups of V columns: col0 + (sl + LPN*u)*V.
+template <int V, int U, int SPLIT>
 struct SweepGeom {
     static constexpr int LPN = 32 / SPLIT;
-    static constexpr int SLAB = LPN * 4 * U;
+    static constexpr int SLAB = LPN * V * U;
 };
 
 // One chunk (up to 32 entries, lane l holds entry l: column k, scalar s) of the Alg. 2 SAXPY
 // sweep.  SRC(j) gives the lane that holds entry j's scalar.
-template <int U, int SPLIT, bool PERMUTED, typename DT>
-__device__ __forceinline__ void saxpy_chunk(float4 (&acc)[U], int k, float s, int cnt,
+template <int V, int U, int SPLIT, bool PERMUTED, typename DT>
+__device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, int cnt,
                                             const DT *__restrict__ Dcol, int64_t ldd,
                                             bool (&live)[U], int sub)
 {
@@ -165,7 +191,7 @@ __device__ __forceinline__ void saxpy_chunk(float4 (&acc)[U], int k, float s, in
             const DT *d = Dcol + (int64_t)kk * ldd;
 #pragma unroll
             for (int u = 0; u < U; ++u)
-                if (live[u]) fma4(acc[u], ss, ldg4(d + u * LPN * 4));
+                if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
         }
     } else {
         for (int jj = 0; jj < STEPS; ++jj) {
@@ -177,15 +203,15 @@ __device__ __forceinline__ void saxpy_chunk(float4 (&acc)[U], int k, float s, in
                 const DT *d = Dcol + (int64_t)kk * ldd;
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (live[u]) fma4(acc[u], ss, ldg4(d + u * LPN * 4));
+                    if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
             }
         }
     }
 }
 
 // Combine the sub-warps of a warp, then the warps of the CTA (fixed order), and store the row.
-template <int U, int SPLIT>
-__device__ __forceinline__ void reduce_and_store_row(float4 (&acc)[U], float4 *red, int warp,
+template <int V, int U, int SPLIT>
+__device__ __forceinline__ void reduce_and_store_row(VecF<V> (&acc)[U], VecF<V> *red, int warp,
                                                      int lane, float *__restrict__ Orow,
                                                      bool (&live)[U])
 {
@@ -194,10 +220,8 @@ __device__ __forceinline__ void reduce_and_store_row(float4 (&acc)[U], float4 *r
     for (int off = 16; off >= LPN; off >>= 1) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            acc[u].x += __shfl_xor_sync(kFull, acc[u].x, off);
-            acc[u].y += __shfl_xor_sync(kFull, acc[u].y, off);
-            acc[u].z += __shfl_xor_sync(kFull, acc[u].z, off);
-            acc[u].w += __shfl_xor_sync(kFull, acc[u].w, off);
+#pragma unroll
+            for (int i = 0; i < V; ++i) acc[u].e[i] += __shfl_xor_sync(kFull, acc[u].e[i], off);
         }
     }
     if (lane < LPN) {
@@ -209,29 +233,30 @@ __device__ __forceinline__ void reduce_and_store_row(float4 (&acc)[U], float4 *r
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (!live[u]) continue;
-            float4 r = red[u * LPN + lane];
+            VecF<V> r = red[u * LPN + lane];
 #pragma unroll
             for (int w = 1; w < kRowWarps; ++w) {
-                float4 t = red[(w * U + u) * LPN + lane];
-                r.x += t.x; r.y += t.y; r.z += t.z; r.w += t.w;
+                const VecF<V> t = red[(w * U + u) * LPN + lane];
+#pragma unroll
+                for (int i = 0; i < V; ++i) r.e[i] += t.e[i];
             }
-            *reinterpret_cast<float4 *>(Orow + u * LPN * 4) = r;
+            *reinterpret_cast<VecF<V> *>(Orow + u * LPN * V) = r;
         }
     }
 }
 
 // ------------------------------------------------------------------------------------------
-// SPMM  (Alg. 2; float4 path: N, ldd, ldo multiples of 4, D and O 16-byte aligned)
+// SPMM  (Alg. 2; N, ldd, ldo multiples of V, D and O aligned to V elements)
 // ------------------------------------------------------------------------------------------
-template <int U, int SPLIT, typename DT>
+template <int V, int U, int SPLIT, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                 const float *__restrict__ values, const DT *__restrict__ D, int64_t ldd,
                 float *__restrict__ O, int64_t ldo, const int *__restrict__ row_order,
                 int *__restrict__ gate, int nrows, int *__restrict__ clear)
 {
-    using G = SweepGeom<U, SPLIT>;
-    __shared__ float4 red[kRowWarps * U * G::LPN];
+    using G = SweepGeom<V, U, SPLIT>;
+    __shared__ VecF<V> red[kRowWarps * U * G::LPN];
     if (gate_closed(gate)) return;
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
@@ -239,13 +264,13 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
     const int sub = lane / G::LPN, sl = lane % G::LPN;
     for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
         const int row = row_order ? row_order[rb] : rb;
-        const int col0 = blockIdx.y * G::SLAB + sl * 4;
+        const int col0 = blockIdx.y * G::SLAB + sl * V;
         bool live[U];
-        float4 acc[U];
+        VecF<V> acc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            live[u] = col0 + u * G::LPN * 4 < N;
-            acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            live[u] = col0 + u * G::LPN * V < N;
+            acc[u] = VecF<V>{};
         }
         const int beg = row_ptr[row], end = row_ptr[row + 1];
         const DT *Dcol = D + col0;
@@ -268,78 +293,26 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
                 kn = __ldg(col_idx + pn);
                 sn = __ldg(values + pn);
             }
-            saxpy_chunk<U, SPLIT, false, DT>(acc, k, s, min(32, end - c), Dcol, ldd, live, sub);
+            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, min(32, end - c), Dcol, ldd, live, sub);
             k = kn;
             s = sn;
         }
-        reduce_and_store_row<U, SPLIT>(acc, red, warp, lane, O + (int64_t)row * ldo + col0, live);
-        __syncthreads();   // shared memory is reused by the next row
-    }
-}
-
-// Scalar path for any N / ld / alignment: a lane owns columns col0 + lane + 32u (u < 4).
-template <typename DT>
-__global__ void __launch_bounds__(kRowThreads)
-spmm_row_scalar_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
-                       const float *__restrict__ values, const DT *__restrict__ D, int64_t ldd,
-                       float *__restrict__ O, int64_t ldo, const int *__restrict__ row_order,
-                       int *__restrict__ gate, int nrows, int *__restrict__ clear)
-{
-    __shared__ float red[kRowWarps][128];
-    if (gate_closed(gate)) return;
-    if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
-    if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
-        const int col0 = blockIdx.y * 128 + lane;
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        const int beg = row_ptr[row], end = row_ptr[row + 1];
-        for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
-            int p = c + lane;
-            int k = 0;
-            float s = 0.f;
-            if (p < end) {
-                k = __ldg(col_idx + p);
-                s = __ldg(values + p);
-            }
-            int cnt = min(32, end - c);
-            for (int j = 0; j < cnt; ++j) {
-                int kk = __shfl_sync(kFull, k, j);
-                float ss = __shfl_sync(kFull, s, j);
-                const DT *d = D + (int64_t)kk * ldd + col0;
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (col0 + 32 * u < N) acc[u] = fmaf(ss, ldg1(d + 32 * u), acc[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) red[warp][lane + 32 * u] = acc[u];
-        __syncthreads();
-        if (warp == 0) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (col0 + 32 * u >= N) continue;
-                float r = red[0][lane + 32 * u];
-                for (int w = 1; w < kRowWarps; ++w) r += red[w][lane + 32 * u];
-                O[(int64_t)row * ldo + col0 + 32 * u] = r;
-            }
-        }
+        reduce_and_store_row<V, U, SPLIT>(acc, red, warp, lane, O + (int64_t)row * ldo + col0, live);
         __syncthreads();   // shared memory is reused by the next row
     }
 }
 
 // ------------------------------------------------------------------------------------------
-// SDDMM  (Alg. 1; float4 path: Kd, lda, ldb multiples of 4, A and B 16-byte aligned)
+// SDDMM  (Alg. 1; Kd, lda, ldb multiples of V, A and B aligned to V elements)
 //
 // A group of 8 lanes computes one sampled dot product: lane t of the group owns elements
-// (t + 8u)*4 .. +3 of the Kd-vector.  KU > 0: A_i is held in KU float4 registers per lane
-// (Kd <= 32*KU).  KU == 0: any Kd, A_i staged in shared memory.  In a chunk of 32 entries,
+// (t + 8u)*V .. +V-1 of the Kd-vector.  KU > 0: A_i is held in KU groups of registers per lane
+// (Kd <= 8*V*KU).  KU == 0: any Kd, A_i staged in shared memory.  In a chunk of 32 entries,
 // group g takes entries 4r + g (r = 0..7); after the 3-step butterfly every lane of the
 // group has the sum and lane t keeps round t's, so lane 8g + t ends up holding entry 4t + g.
 // ------------------------------------------------------------------------------------------
-template <int KU, typename DT>
-__device__ __forceinline__ float sddmm_chunk(const float4 (&areg)[KU > 0 ? KU : 1],
+template <int V, int KU, typename DT>
+__device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU : 1],
                                              const float *__restrict__ a_smem, int Kd, int k,
                                              const DT *__restrict__ B, int64_t ldb, int lane)
 {
@@ -348,15 +321,15 @@ __device__ __forceinline__ float sddmm_chunk(const float4 (&areg)[KU > 0 ? KU : 
 #pragma unroll 4
     for (int r = 0; r < 8; ++r) {
         int kq = __shfl_sync(kFull, k, 4 * r + g);
-        const DT *b = B + (int64_t)kq * ldb + t * 4;
+        const DT *b = B + (int64_t)kq * ldb + t * V;
         float part = 0.f;
         if (KU > 0) {
 #pragma unroll
             for (int u = 0; u < KU; ++u)
-                if ((t + 8 * u) * 4 < Kd) part = dot4(areg[u], ldg4(b + u * 32), part);
+                if ((t + 8 * u) * V < Kd) part = dot_v<V>(areg[u], ldgv<V>(b + u * 8 * V), part);
         } else {
-            for (int e = t * 4; e < Kd; e += 32)
-                part = dot4(*reinterpret_cast<const float4 *>(a_smem + e), ldg4(b + e - t * 4), part);
+            for (int e = t * V; e < Kd; e += 8 * V)
+                part = dot_v<V>(*reinterpret_cast<const VecF<V> *>(a_smem + e), ldgv<V>(b + e - t * V), part);
         }
         part += __shfl_xor_sync(kFull, part, 1);
         part += __shfl_xor_sync(kFull, part, 2);
@@ -366,23 +339,23 @@ __device__ __forceinline__ float sddmm_chunk(const float4 (&areg)[KU > 0 ? KU : 
     return mine;  // lane 8g+t: dot product of entry 4t+g
 }
 
-template <int KU, typename DT>
-__device__ __forceinline__ void load_a_row(float4 (&areg)[KU > 0 ? KU : 1], float *a_smem,
+template <int V, int KU, typename DT>
+__device__ __forceinline__ void load_a_row(VecF<V> (&areg)[KU > 0 ? KU : 1], float *a_smem,
                                            const DT *__restrict__ Arow, int Kd, int lane)
 {
     if (KU > 0) {
         const int t = lane & 7;
 #pragma unroll
         for (int u = 0; u < (KU > 0 ? KU : 1); ++u)
-            areg[u] = (t + 8 * u) * 4 < Kd ? ldg4(Arow + (t + 8 * u) * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            areg[u] = (t + 8 * u) * V < Kd ? ldgv<V>(Arow + (t + 8 * u) * V) : VecF<V>{};
     } else {
-        for (int e = threadIdx.x * 4; e < Kd; e += kRowThreads * 4)
-            *reinterpret_cast<float4 *>(a_smem + e) = ldg4(Arow + e);
+        for (int e = threadIdx.x * V; e < Kd; e += kRowThreads * V)
+            *reinterpret_cast<VecF<V> *>(a_smem + e) = ldgv<V>(Arow + e);
         __syncthreads();
     }
 }
 
-template <int KU, typename DT>
+template <int V, int KU, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                  const float *s_values, const DT *__restrict__ A, int64_t lda,
@@ -398,13 +371,13 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
     for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
         const int row = row_order ? row_order[rb] : rb;
         const int beg = row_ptr[row], end = row_ptr[row + 1];
-        float4 areg[KU > 0 ? KU : 1];
-        load_a_row<KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
+        VecF<V> areg[KU > 0 ? KU : 1];
+        load_a_row<V, KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
         const int slot = (lane & 7) * 4 + (lane >> 3);  // entry of the chunk this lane ends up holding
         for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
             int p = c + lane;
             int k = p < end ? __ldg(col_idx + p) : 0;
-            float dp = sddmm_chunk<KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
+            float dp = sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
             int q = c + slot;
             if (q < end) out_values[q] = s_values ? s_values[q] * dp : dp;
         }
@@ -412,7 +385,7 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
     }
 }
 
-// Scalar path for any Kd / ld / alignment: one lane per entry, serial dot product.
+// Kd too long for A_i in shared memory (kMaxStagedKd): one lane per entry, serial dot product.
 template <typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 sddmm_row_scalar_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
@@ -441,7 +414,7 @@ sddmm_row_scalar_kernel(int Kd, const int *__restrict__ row_ptr, const int *__re
 // FusedMM  (Alg. 3): per chunk, the SDDMM values stay in registers (one per lane) and are the
 // scalars of the SAXPY sweep over the same staged column indices; C never reaches memory.
 // ------------------------------------------------------------------------------------------
-template <int KU, int U, int SPLIT, bool BATCHED, typename DT>
+template <int V, int KU, int U, int SPLIT, bool BATCHED, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                    const float *__restrict__ s_values, const DT *__restrict__ A, int64_t lda,
@@ -450,7 +423,7 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
                    const int *__restrict__ row_order, int *__restrict__ gate, int nrows, int *__restrict__ clear,
                    typename BatchArg<BATCHED>::type batch)
 {
-    using G = SweepGeom<U, SPLIT>;
+    using G = SweepGeom<V, U, SPLIT>;
     extern __shared__ float4 dyn_smem[];
     if (gate_closed(gate)) return;
     if constexpr (BATCHED) {   // this problem's arrays
@@ -460,23 +433,23 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
     }
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
-    float4 *red = dyn_smem;                                                   // kRowWarps*U*LPN
-    float *a_smem = reinterpret_cast<float *>(dyn_smem + kRowWarps * U * G::LPN);  // Kd (KU == 0)
+    VecF<V> *red = reinterpret_cast<VecF<V> *>(dyn_smem);                // kRowWarps*U*LPN
+    float *a_smem = reinterpret_cast<float *>(red + kRowWarps * U * G::LPN);  // Kd (KU == 0)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / G::LPN, sl = lane % G::LPN;
     for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
         const int row = row_order ? row_order[rb] : rb;
-        const int col0 = blockIdx.y * G::SLAB + sl * 4;
+        const int col0 = blockIdx.y * G::SLAB + sl * V;
         bool live[U];
-        float4 acc[U];
+        VecF<V> acc[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            live[u] = col0 + u * G::LPN * 4 < N;
-            acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            live[u] = col0 + u * G::LPN * V < N;
+            acc[u] = VecF<V>{};
         }
         const int beg = row_ptr[row], end = row_ptr[row + 1];
-        float4 areg[KU > 0 ? KU : 1];
-        load_a_row<KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
+        VecF<V> areg[KU > 0 ? KU : 1];
+        load_a_row<V, KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
         const int slot = (lane & 7) * 4 + (lane >> 3);
         const DT *Dcol = D + col0;
         int k = 0;
@@ -490,17 +463,17 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
             int pn = c + kRowWarps * 32 + lane, qn = c + kRowWarps * 32 + slot;
             int kn = pn < end ? __ldg(col_idx + pn) : 0;
             float svn = (s_values && qn < end) ? __ldg(s_values + qn) : 1.f;
-            float cv = sv * sddmm_chunk<KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
-            saxpy_chunk<U, SPLIT, true, DT>(acc, k, cv, min(32, end - c), Dcol, ldd, live, sub);
+            float cv = sv * sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
+            saxpy_chunk<V, U, SPLIT, true, DT>(acc, k, cv, min(32, end - c), Dcol, ldd, live, sub);
             k = kn;
             sv = svn;
         }
-        reduce_and_store_row<U, SPLIT>(acc, red, warp, lane, O + (int64_t)row * ldo + col0, live);
+        reduce_and_store_row<V, U, SPLIT>(acc, red, warp, lane, O + (int64_t)row * ldo + col0, live);
         __syncthreads();   // shared memory is reused by the next row
     }
 }
 
-// Scalar path for any widths / alignment: lane-per-entry dot products, then a scalar sweep.
+// Kd too long for A_i in shared memory: lane-per-entry dot products, then a scalar sweep.
 template <typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 fusedmm_row_scalar_kernel(int Kd, int N, const int *__restrict__ row_ptr,
