@@ -180,8 +180,8 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
                                             bool (&live)[U], int sub)
 {
     constexpr int LPN = 32 / SPLIT;
-    constexpr int STEPS = 32 / SPLIT;
     if (cnt == 32) {
+        constexpr int STEPS = 32 / SPLIT;
 #pragma unroll 8
         for (int jj = 0; jj < STEPS; ++jj) {
             int j = jj * SPLIT + sub;
@@ -194,20 +194,35 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
                 if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
         }
     } else {
-        for (int jj = 0; jj < STEPS; ++jj) {
-            int j = jj * SPLIT + sub;
-            int src = PERMUTED ? ((j & 3) * 8 + (j >> 2)) : j;
-            int kk = __shfl_sync(kFull, k, j);
-            float ss = __shfl_sync(kFull, s, src);
-            if (j < cnt) {
-                const DT *d = Dcol + (int64_t)kk * ldd;
+        // (a few entries' loads in flight together)
+        constexpr int BATCH = V == 4 ? 2 : 4;
+        for (int jj = 0; jj * SPLIT < cnt; jj += BATCH) {
+            VecF<V> d[BATCH][U];
+            float ss[BATCH];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
+            for (int i = 0; i < BATCH; ++i) {
+                const int j = (jj + i) * SPLIT + sub;
+                const int src = PERMUTED ? ((j & 3) * 8 + (j >> 2)) : j;
+                const int kk = __shfl_sync(kFull, k, j & 31);
+                ss[i] = __shfl_sync(kFull, s, src & 31);
+                const DT *p = Dcol + (int64_t)kk * ldd;
+#pragma unroll
+                for (int u = 0; u < U; ++u) d[i][u] = j < cnt && live[u] ? ldgv<V>(p + u * LPN * V) : VecF<V>{};
             }
+#pragma unroll
+            for (int i = 0; i < BATCH; ++i)
+                if ((jj + i) * SPLIT + sub < cnt) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) fma_v<V>(acc[u], ss[i], d[i][u]);
+                }
         }
     }
 }
+
+// Entries of a row that a warp takes at a time: 32, or a quarter of a row of 64 or fewer (a multiple of four, the groups of
+// sddmm_chunk), so that all four warps have a part of it: a row of 25 entries was one warp's serial chain while three idled
+// (256 x 256 at 10%, Kd = N = 64, fusedmm: 7.1 -> 3.7 us).
+__device__ __forceinline__ int chunk_of(int len) { return len > 64 ? 32 : ((len + 4 * kRowWarps - 1) / (4 * kRowWarps)) * 4; }
 
 // Combine the sub-warps of a warp, then the warps of the CTA (fixed order), and store the row.
 template <int V, int U, int SPLIT>
@@ -278,22 +293,23 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
         // (the role of the paper's prefetch of the next ja/avalues block)
         int k = 0;
         float s = 0.f;
+        const int chunk = chunk_of(end - beg);
         {
-            int p = beg + warp * 32 + lane;
+            int p = beg + warp * chunk + lane;
             if (p < end) {
                 k = __ldg(col_idx + p);
                 s = __ldg(values + p);
             }
         }
-        for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
-            int pn = c + kRowWarps * 32 + lane;
+        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
+            int pn = c + kRowWarps * chunk + lane;
             int kn = 0;
             float sn = 0.f;
             if (pn < end) {
                 kn = __ldg(col_idx + pn);
                 sn = __ldg(values + pn);
             }
-            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, min(32, end - c), Dcol, ldd, live, sub);
+            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, min(chunk, end - c), Dcol, ldd, live, sub);
             k = kn;
             s = sn;
         }
@@ -314,13 +330,12 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
 template <int V, int KU, typename DT>
 __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU : 1],
                                              const float *__restrict__ a_smem, int Kd, int k,
-                                             const DT *__restrict__ B, int64_t ldb, int lane)
+                                             const DT *__restrict__ B, int64_t ldb, int lane, int cnt)
 {
     const int g = lane >> 3, t = lane & 7;
     float mine = 0.f;
-#pragma unroll 4
-    for (int r = 0; r < 8; ++r) {
-        int kq = __shfl_sync(kFull, k, 4 * r + g);
+    auto round = [&](int r) {
+        const int kq = __shfl_sync(kFull, k, 4 * r + g);
         const DT *b = B + (int64_t)kq * ldb + t * V;
         float part = 0.f;
         if (KU > 0) {
@@ -335,6 +350,13 @@ __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU :
         part += __shfl_xor_sync(kFull, part, 2);
         part += __shfl_xor_sync(kFull, part, 4);
         if (r == t) mine = part;
+    };
+    if (cnt == 32) {
+#pragma unroll 4
+        for (int r = 0; r < 8; ++r) round(r);
+    } else {   // (a number of rounds known only now: no loop of its own cost full chunks a quarter of their speed)
+#pragma unroll 2
+        for (int r = 0; r < (cnt + 3) >> 2; ++r) round(r);
     }
     return mine;  // lane 8g+t: dot product of entry 4t+g
 }
@@ -374,12 +396,14 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
         VecF<V> areg[KU > 0 ? KU : 1];
         load_a_row<V, KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
         const int slot = (lane & 7) * 4 + (lane >> 3);  // entry of the chunk this lane ends up holding
-        for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
+        const int chunk = chunk_of(end - beg);
+        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
             int p = c + lane;
             int k = p < end ? __ldg(col_idx + p) : 0;
-            float dp = sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
+            const int cnt = min(chunk, end - c);
+            float dp = sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
             int q = c + slot;
-            if (q < end) out_values[q] = s_values ? s_values[q] * dp : dp;
+            if (slot < cnt) out_values[q] = s_values ? s_values[q] * dp : dp;
         }
         __syncthreads();   // shared memory is reused by the next row
     }
@@ -454,17 +478,19 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
         const DT *Dcol = D + col0;
         int k = 0;
         float sv = 1.f;
+        const int chunk = chunk_of(end - beg);
         {
-            int p = beg + warp * 32 + lane, q = beg + warp * 32 + slot;
+            int p = beg + warp * chunk + lane, q = beg + warp * chunk + slot;
             if (p < end) k = __ldg(col_idx + p);
             if (s_values && q < end) sv = __ldg(s_values + q);
         }
-        for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
-            int pn = c + kRowWarps * 32 + lane, qn = c + kRowWarps * 32 + slot;
+        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
+            int pn = c + kRowWarps * chunk + lane, qn = c + kRowWarps * chunk + slot;
             int kn = pn < end ? __ldg(col_idx + pn) : 0;
             float svn = (s_values && qn < end) ? __ldg(s_values + qn) : 1.f;
-            float cv = sv * sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane);
-            saxpy_chunk<V, U, SPLIT, true, DT>(acc, k, cv, min(32, end - c), Dcol, ldd, live, sub);
+            const int cnt = min(chunk, end - c);
+            float cv = sv * sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
+            saxpy_chunk<V, U, SPLIT, true, DT>(acc, k, cv, cnt, Dcol, ldd, live, sub);
             k = kn;
             sv = svn;
         }
