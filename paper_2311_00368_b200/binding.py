@@ -11,6 +11,7 @@ Function names and argument order follow ``include/b2sp.h`` (and ``include/b2sp_
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import torch
@@ -101,23 +102,33 @@ def _check(status: int, where: str):
         raise B2spError(status, where)
 
 
+# The argument marshalling is on the critical path of small calls (a few microseconds of GPU work): addresses and streams are
+# passed as plain integers, which the declared argument types convert, and the stream is asked for without a Stream object.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+try:
+    _raw_stream = torch._C._cuda_getCurrentRawStream   # device index -> cudaStream_t of torch's current stream
+except AttributeError:
+    def _raw_stream(device_index):
+        return torch.cuda.current_stream(device_index).cuda_stream
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _ld(t):
-    assert t.dim() == 2 and (t.shape[1] <= 1 or t.stride(1) == 1), "dense operands are row-major"
-    return t.stride(0) if t.shape[0] > 1 else max(t.shape[1], t.stride(0))
+    shape, strides = t.shape, t.stride()
+    assert len(shape) == 2 and (shape[1] <= 1 or strides[1] == 1), "dense operands are row-major"
+    return strides[0] if shape[0] > 1 else max(shape[1], strides[0])
 
 
 def _want(t, dtype, name, cuda=True):
     if t is None:
         return
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}")
     if cuda and not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
@@ -137,10 +148,16 @@ def workspace_bytes(op: int, M: int, K: int, Kd: int, N: int, nnz: int, algo=Non
 _ws_cache = {}
 
 
+# Sizes only; emptied by the debug hooks that change the planner's choice.
+@functools.lru_cache(maxsize=4096)
+def _workspace_need(op, M, K, Kd, N, nnz, algo):
+    return workspace_bytes(op, M, K, Kd, N, nnz, algo)
+
+
 def _workspace(op, M, K, Kd, N, nnz, device, workspace, algo=0):
     if workspace is None:
-        need = workspace_bytes(op, M, K, Kd, N, nnz, algo)
-        key = (device.index, torch.cuda.current_stream(device).cuda_stream)
+        need = _workspace_need(op, M, K, Kd, N, nnz, algo)
+        key = (device.index, _raw_stream(device.index))
         workspace = _ws_cache.get(key)
         if workspace is None or workspace.numel() < need:
             workspace = torch.empty(max(need, 1 << 20), dtype=torch.uint8, device=device)
@@ -175,11 +192,13 @@ def last_launches(op: int) -> int:
 
 def debug_force_k_splits(k_splits: int) -> None:
     """b2sp_debug_force_k_splits: override the dense-tile planner's K split (0 = planner's choice)."""
+    _workspace_need.cache_clear()
     lib.b2sp_debug_force_k_splits(int(k_splits))
 
 
 def debug_force_partition(partition: int) -> None:
     """b2sp_debug_force_partition: 0 = planner's choice, 1 = tiles x K splits only, 2 = balanced wherever offered."""
+    _workspace_need.cache_clear()
     lib.b2sp_debug_force_partition(int(partition))
 
 
