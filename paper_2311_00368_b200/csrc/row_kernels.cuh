@@ -194,7 +194,8 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
                 if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
         }
     } else {
-        // (a few entries' loads in flight together)
+        // (a few entries' loads in flight together; four of four-element groups take registers that the full chunks miss:
+        // 3072 x 1024 x 32 7.2 -> 7.5 us; two of single elements are too few: 1501 x 2903 x 71 24.8 -> 27.5 us)
         constexpr int BATCH = V == 4 ? 2 : 4;
         for (int jj = 0; jj * SPLIT < cnt; jj += BATCH) {
             VecF<V> d[BATCH][U];
@@ -221,7 +222,8 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
 
 // Entries of a row that a warp takes at a time: 32, or a quarter of a row of 64 or fewer (a multiple of four, the groups of
 // sddmm_chunk), so that all four warps have a part of it: a row of 25 entries was one warp's serial chain while three idled
-// (256 x 256 at 10%, Kd = N = 64, fusedmm: 7.1 -> 3.7 us).
+// (256 x 256 at 10%, Kd = N = 64, fusedmm: 7.1 -> 4.0 us; 4096 x 512 at 5%, Kd = 100, N = 250: 83 -> 32 us).  With the line at
+// 128 entries, rows of 102 lost their full chunks' eight loads in flight (3072 x 1024 x 32 spmm 7.1 -> 7.5 us).
 __device__ __forceinline__ int chunk_of(int len) { return len > 64 ? 32 : ((len + 4 * kRowWarps - 1) / (4 * kRowWarps)) * 4; }
 
 // Combine the sub-warps of a warp, then the warps of the CTA (fixed order), and store the row.
@@ -354,7 +356,7 @@ __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU :
     if (cnt == 32) {
 #pragma unroll 4
         for (int r = 0; r < 8; ++r) round(r);
-    } else {   // (a number of rounds known only now: no loop of its own cost full chunks a quarter of their speed)
+    } else {   // (one loop for both, its length known only at run time, cost full chunks a quarter of their speed)
 #pragma unroll 2
         for (int r = 0; r < (cnt + 3) >> 2; ++r) round(r);
     }
