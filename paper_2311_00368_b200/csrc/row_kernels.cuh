@@ -194,9 +194,11 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
                 if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
         }
     } else {
-        // (a few entries' loads in flight together; four of four-element groups take registers that the full chunks miss:
-        // 3072 x 1024 x 32 7.2 -> 7.5 us; two of single elements are too few: 1501 x 2903 x 71 24.8 -> 27.5 us)
-        constexpr int BATCH = V == 4 ? 2 : 4;
+        // Entries whose loads are in flight together.  It is a matter of registers, which the full chunks then miss, and was
+        // measured: single or pair elements four (two: 1501 x 2903 x 71 spmm 24.8 -> 27.5 us); SPMM with whole warps two (one:
+        // 8192 x 8192 at 10% x 256 385 -> 514 us, x 128 248 -> 298 us); FusedMM and sub-warps one (two: 4096 x 4096 at 20% x 64
+        // spmm 69 -> 74 us, 8192 x 8192 at 5%, Kd = N = 32, fusedmm 90 -> 97 us).
+        constexpr int BATCH = V < 4 ? 4 : !PERMUTED && SPLIT == 1 ? 2 : 1;
         for (int jj = 0; jj * SPLIT < cnt; jj += BATCH) {
             VecF<V> d[BATCH][U];
             float ss[BATCH];
