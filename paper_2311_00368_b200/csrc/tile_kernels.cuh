@@ -15,6 +15,7 @@
 #include <stdint.h>
 
 #include "ptx_sm100.cuh"
+#include "row_walk.h"
 #include "tile_dispatch.h"
 
 namespace b2sp {
@@ -44,8 +45,6 @@ constexpr int kPatternMagic = 0x62327370;
 // windows (a prefix sum over the pop counts).  Every window of every row is written, so the table needs no clearing.
 // The table is only meaningful when the columns of each row are strictly increasing and in range;
 // the first sweep checks exactly that and sets flags[kFlagUnsorted] if not.
-constexpr int kMasksRun = 8;                          // consecutive entries of a lane
-constexpr int kMasksChunk = 32 * kMasksRun;           // entries of a warp's iteration
 constexpr int kMasksMaxWk = 24 * 1024;                // the mask row must fit in the shared memory a block may ask for (96 KB)
 constexpr int kMasksMaxSmem = kMasksMaxWk * 4;
 constexpr int kMasksRows = 8;                         // rows (= warps) of a tile_masks_kernel<false> block
@@ -53,12 +52,12 @@ constexpr int kMasksOwn = 2048;                       // entries of its row that
 constexpr int kMasksSharedWarps = 4;                  // warps of a tile_masks_kernel<true> block
 __host__ __device__ constexpr int masks_row_words(int Wk) { return (Wk + 127) & ~127; }   // (cleared sixteen bytes per lane)
 
-// Entries p .. p + 7 of a row [beg, end): sixteen-byte loads where all of them are inside the array (p is chosen so that
-// their addresses are aligned), single ones of the row otherwise.
-__device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, int nnz, int beg, int end, int p, int (&v)[kMasksRun])
+// Entries p .. p + 7: sixteen-byte loads where all of them may be read (p is chosen so that their addresses are aligned), single
+// ones of the row otherwise.
+__device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, const TableRow &row, int p, int (&v)[kMasksRun])
 {
-    if (p >= end) return;
-    if (p >= 0 && p <= nnz - kMasksRun) {
+    if (p >= row.end) return;
+    if (row.wide(p)) {
 #pragma unroll
         for (int i = 0; i < kMasksRun; i += 4) {
             const int4 x = __ldg(reinterpret_cast<const int4 *>(col_idx + p + i));
@@ -67,7 +66,7 @@ __device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, 
     } else {
 #pragma unroll
         for (int i = 0; i < kMasksRun; ++i)
-            if (p + i >= beg && p + i < end) v[i] = __ldg(col_idx + p + i);
+            if (row.has(p + i)) v[i] = __ldg(col_idx + p + i);
     }
 }
 
@@ -145,13 +144,14 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
         const int *__restrict__ col_idx = col_idx0 + pb * sig.nz_stride;
         const int beg = live ? __ldg(row_ptr + row) : 0, end = live ? __ldg(row_ptr + row + 1) : 0;
         int c[kMasksRun], c_next[kMasksRun];
-        // where lane 0 of the row's first run begins: at or up to three entries before the row, so that loads are aligned
-        const int first = beg - ((beg + ((int)(reinterpret_cast<uintptr_t>(col_idx) >> 2) & 3)) & 3);
+        const unsigned misalign = (unsigned)(reinterpret_cast<uintptr_t>(col_idx) >> 2) & 3u;
+        const TableRow tr(beg, end, load_limit(end, pb, sig.batch, nnz), misalign);
+        const int first = tr.first;
         const int own_end = SHARED ? end : (end - first > kMasksOwn ? first + kMasksOwn : end);
 #pragma unroll
         for (int i = 0; i < kMasksRun; ++i) c_next[i] = 0;
         int p0 = first + (SHARED ? kMasksChunk * warp : 0);
-        if (beg < end) masks_load_run(col_idx, (int)nnz, beg, end, p0 + kMasksRun * lane, c_next);
+        if (beg < end) masks_load_run(col_idx, tr, p0 + kMasksRun * lane, c_next);
         else p0 = own_end;
         for (int w = (SHARED ? (int)threadIdx.x : lane) * 4; w < words; w += WARPS * 128)
             *reinterpret_cast<uint4 *>(mask + w) = make_uint4(0u, 0u, 0u, 0u);
@@ -163,7 +163,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
             const int p = p0 + kMasksRun * lane;
 #pragma unroll
             for (int i = 0; i < kMasksRun; ++i) c[i] = c_next[i];
-            if (p0 + kMasksChunk * WARPS < own_end) masks_load_run(col_idx, (int)nnz, beg, end, p + kMasksChunk * WARPS, c_next);
+            if (p0 + kMasksChunk * WARPS < own_end) masks_load_run(col_idx, tr, p + kMasksChunk * WARPS, c_next);
             int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
             if (lane == 0) prev = !SHARED ? carry : p > beg ? __ldg(col_idx + p - 1) : 0;
             if (!SHARED) carry = __shfl_sync(kFull, c[kMasksRun - 1], 31);
@@ -178,10 +178,11 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
                 const int4 q = rest[r];
                 if (q.z >= q.w) continue;
                 const int *__restrict__ ci = col_idx0 + q.x * sig.nz_stride;
+                const TableRow other(q.y, q.w, q.w, 0);
                 const int chunks = (q.w - q.z + kMasksChunk - 1) / kMasksChunk;
                 for (int j = (warp - turn) & (ROWS - 1); j < chunks; j += ROWS) {
                     const int pc = q.z + j * kMasksChunk, p = pc + kMasksRun * lane;
-                    masks_load_run(ci, (int)nnz, q.y, q.w, p, c);
+                    masks_load_run(ci, other, p, c);
                     int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
                     if (lane == 0) prev = __ldg(ci + p - 1);
                     bad |= !masks_or_run(c, prev, p, q.y, q.w, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
