@@ -48,24 +48,24 @@ constexpr int kPatternMagic = 0x62327370;
 constexpr int kMasksMaxWk = 24 * 1024;                // the mask row must fit in the shared memory a block may ask for (96 KB)
 constexpr int kMasksMaxSmem = kMasksMaxWk * 4;
 constexpr int kMasksRows = 8;                         // rows (= warps) of a tile_masks_kernel<false> block
-constexpr int kMasksOwn = 2048;                       // entries of its row that a warp of such a block reads by itself
+constexpr unsigned kMasksOwn = 2048;                       // entries of its row that a warp of such a block reads by itself
 constexpr int kMasksSharedWarps = 4;                  // warps of a tile_masks_kernel<true> block
 __host__ __device__ constexpr int masks_row_words(int Wk) { return (Wk + 127) & ~127; }   // (cleared sixteen bytes per lane)
 
 // Entries p .. p + 7: sixteen-byte loads where all of them may be read (p is chosen so that their addresses are aligned), single
 // ones of the row otherwise.
-__device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, const TableRow &row, int p, int (&v)[kMasksRun])
+__device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, const TableRow &row, unsigned p, int (&v)[kMasksRun])
 {
     if (p >= row.end) return;
     if (row.wide(p)) {
 #pragma unroll
-        for (int i = 0; i < kMasksRun; i += 4) {
+        for (unsigned i = 0; i < kMasksRun; i += 4) {
             const int4 x = __ldg(reinterpret_cast<const int4 *>(col_idx + p + i));
             v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kMasksRun; ++i)
+        for (unsigned i = 0; i < kMasksRun; ++i)
             if (row.has(p + i)) v[i] = __ldg(col_idx + p + i);
     }
 }
@@ -74,11 +74,11 @@ __device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, 
 // entry before the run, `interior` (the same for the whole warp): every lane's run is inside the row.  false: the row is not
 // strictly increasing or out of range (a table with such a row is not used).  Neighbouring lanes are eight entries apart,
 // so that they hardly ever OR into the same word at the same time (consecutive entries mostly share one).
-__device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev, int p, int beg, int end, int K, uint32_t words, bool interior)
+__device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev, unsigned p, const TableRow &row, int K, uint32_t words, bool interior)
 {
     auto or_bit = [&](int col) { ptx::red_or_shared(words + 4 * (col >> 5), __funnelshift_l(0u, 1u, col)); };   // 1 << (column within the window)
     if (interior) {
-        bool ok = (p <= beg || c[0] > prev) && c[0] >= 0 && c[kMasksRun - 1] < K;   // (in order, so the others are in range too)
+        bool ok = (p <= row.beg || c[0] > prev) && c[0] >= 0 && c[kMasksRun - 1] < K;   // (in order, so the others are in range too)
 #pragma unroll
         for (int i = 1; i < kMasksRun; ++i) ok = ok && c[i] > c[i - 1];
         if (!ok) return false;
@@ -86,13 +86,12 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
         for (int i = 0; i < kMasksRun; ++i) or_bit(c[i]);
         return true;
     }
-    const int at = p - beg, len = end - beg;   // an end of the row: entries at .. at + 7 of it, some of them not in it
-    bool bad = false;
+    bool bad = false;   // an end of the row: some of the entries are not in it
 #pragma unroll
     for (int i = 0; i < kMasksRun; ++i) {
-        if ((unsigned)(at + i) >= (unsigned)len) continue;
+        if (!row.has(p + i)) continue;
         const bool in_range = (unsigned)c[i] < (unsigned)K;
-        bad |= !in_range || (at + i > 0 && c[i] <= (i == 0 ? prev : c[i == 0 ? 0 : i - 1]));
+        bad |= !in_range || (p + i != row.beg && c[i] <= (i == 0 ? prev : c[i == 0 ? 0 : i - 1]));
         if (in_range) or_bit(c[i]);
     }
     return !bad;
@@ -127,7 +126,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
     constexpr int WARPS = SHARED ? kMasksSharedWarps : 1;       // warps of a row
     constexpr int ROWS = SHARED ? 1 : kMasksRows;               // rows of the block at a time
     __shared__ int warp_total[WARPS];
-    __shared__ int4 rest[ROWS];                                 // of each row: problem, first entry, first entry not read yet, end
+    __shared__ uint4 rest[ROWS];                                // of each row: problem, first entry, first entry not read yet, end
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int words = masks_row_words(Wk);
     unsigned *mask = mask_rows + (SHARED ? 0 : warp * words);
@@ -141,51 +140,54 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
         const int pb = sig.batch == 1 || !live ? 0 : rows_all < 0x7fffffffll ? (int)((unsigned)rowg / (unsigned)M) : (int)(rowg / M);
         const int row = live ? (int)(rowg - (long long)pb * M) : 0;
         const int *__restrict__ row_ptr = row_ptr0 + pb * sig.rp_stride;
-        const int *__restrict__ col_idx = col_idx0 + pb * sig.nz_stride;
+        // (from the 16-byte boundary at or before the problem's first entry, see row_walk.h)
+        auto aligned_down = [](const int *p) { return reinterpret_cast<const int *>(reinterpret_cast<uintptr_t>(p) & ~uintptr_t(15)); };
+        auto misalignment = [](const int *p) { return (unsigned)(reinterpret_cast<uintptr_t>(p) >> 2) & 3u; };
+        const int *__restrict__ col_idx = aligned_down(col_idx0 + pb * sig.nz_stride);
+        const unsigned misalign = misalignment(col_idx0 + pb * sig.nz_stride);
         const int beg = live ? __ldg(row_ptr + row) : 0, end = live ? __ldg(row_ptr + row + 1) : 0;
+        const TableRow tr{(unsigned)beg + misalign, (unsigned)end + misalign, load_limit((unsigned)end + misalign, pb, (int)sig.batch, (unsigned)nnz)};
         int c[kMasksRun], c_next[kMasksRun];
-        const unsigned misalign = (unsigned)(reinterpret_cast<uintptr_t>(col_idx) >> 2) & 3u;
-        const TableRow tr(beg, end, load_limit(end, pb, sig.batch, nnz), misalign);
-        const int first = tr.first;
-        const int own_end = SHARED ? end : (end - first > kMasksOwn ? first + kMasksOwn : end);
+        unsigned p0 = tr.first();
+        const unsigned own_end = SHARED || tr.end - p0 <= kMasksOwn ? tr.end : p0 + kMasksOwn;
 #pragma unroll
         for (int i = 0; i < kMasksRun; ++i) c_next[i] = 0;
-        int p0 = first + (SHARED ? kMasksChunk * warp : 0);
+        if (SHARED) p0 += kMasksChunk * warp;
         if (beg < end) masks_load_run(col_idx, tr, p0 + kMasksRun * lane, c_next);
         else p0 = own_end;
         for (int w = (SHARED ? (int)threadIdx.x : lane) * 4; w < words; w += WARPS * 128)
             *reinterpret_cast<uint4 *>(mask + w) = make_uint4(0u, 0u, 0u, 0u);
-        if (!SHARED && lane == 0) rest[warp] = make_int4(pb, beg, beg < end ? own_end : end, end);
+        if (!SHARED && lane == 0) rest[warp] = make_uint4((unsigned)pb, tr.beg, beg < end ? own_end : tr.end, tr.end);
         if (SHARED) __syncthreads();
         else __syncwarp();
         int carry = 0;   // the last entry of the warp's previous iteration
         for (; p0 < own_end; p0 += kMasksChunk * WARPS) {
-            const int p = p0 + kMasksRun * lane;
+            const unsigned p = p0 + kMasksRun * lane;
 #pragma unroll
             for (int i = 0; i < kMasksRun; ++i) c[i] = c_next[i];
             if (p0 + kMasksChunk * WARPS < own_end) masks_load_run(col_idx, tr, p + kMasksChunk * WARPS, c_next);
             int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
-            if (lane == 0) prev = !SHARED ? carry : p > beg ? __ldg(col_idx + p - 1) : 0;
+            if (lane == 0) prev = !SHARED ? carry : p > tr.beg ? __ldg(col_idx + p - 1) : 0;
             if (!SHARED) carry = __shfl_sync(kFull, c[kMasksRun - 1], 31);
-            bad |= !masks_or_run(c, prev, p, beg, end, K, mask_smem, p0 >= beg && p0 + kMasksChunk <= end);
+            bad |= !masks_or_run(c, prev, p, tr, K, mask_smem, p0 >= tr.beg && p0 + kMasksChunk <= tr.end);
         }
         if (SHARED) {
             __syncthreads();
-        } else if (__syncthreads_or(beg < end && own_end < end)) {
+        } else if (__syncthreads_or(beg < end && own_end < tr.end)) {
             // some of the block's rows are longer: their other entries, in chunks dealt to the warps in turn
-            int turn = 0;   // chunks of the rows before
+            unsigned turn = 0;   // chunks of the rows before
             for (int r = 0; r < ROWS; ++r) {
-                const int4 q = rest[r];
+                const uint4 q = rest[r];
                 if (q.z >= q.w) continue;
-                const int *__restrict__ ci = col_idx0 + q.x * sig.nz_stride;
-                const TableRow other(q.y, q.w, q.w, 0);
-                const int chunks = (q.w - q.z + kMasksChunk - 1) / kMasksChunk;
-                for (int j = (warp - turn) & (ROWS - 1); j < chunks; j += ROWS) {
-                    const int pc = q.z + j * kMasksChunk, p = pc + kMasksRun * lane;
+                const int *__restrict__ ci = aligned_down(col_idx0 + q.x * sig.nz_stride);
+                const TableRow other{q.y, q.w, q.w};
+                const unsigned chunks = (q.w - q.z + kMasksChunk - 1) / kMasksChunk;
+                for (unsigned j = (warp - turn) & (ROWS - 1); j < chunks; j += ROWS) {
+                    const unsigned pc = q.z + j * kMasksChunk, p = pc + kMasksRun * lane;
                     masks_load_run(ci, other, p, c);
                     int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
                     if (lane == 0) prev = __ldg(ci + p - 1);
-                    bad |= !masks_or_run(c, prev, p, q.y, q.w, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
+                    bad |= !masks_or_run(c, prev, p, other, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
                 }
                 turn += chunks;
             }

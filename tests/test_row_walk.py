@@ -17,18 +17,41 @@ using namespace b2sp;
 // that is loaded; 0: one outside [0, count).
 extern "C" int table_row(const int *row_ptr, int row, long long nnz, int batch, int last, unsigned misalign, int count, unsigned char *loads)
 {
-    const int beg = row_ptr[row], end = row_ptr[row + 1];
-    const TableRow tr(beg, end, load_limit(end, last ? batch - 1 : 0, batch, nnz), misalign);
-    for (int p0 = tr.first; p0 < tr.end; p0 += kMasksChunk)
+    const unsigned end = row_ptr[row + 1] + misalign;
+    const TableRow tr{row_ptr[row] + misalign, end, load_limit(end, last ? batch - 1 : 0, batch, nnz)};
+    for (unsigned p0 = tr.first(); p0 < tr.end; p0 += kMasksChunk)
         for (int lane = 0; lane < 32; ++lane) {
-            const int p = p0 + kMasksRun * lane;
+            const unsigned p = p0 + kMasksRun * lane;
             if (p >= tr.end) break;
-            for (int i = 0; i < kMasksRun; ++i)
+            for (unsigned i = 0; i < kMasksRun; ++i)
                 if (tr.wide(p) || tr.has(p + i)) {
-                    if (p + i < 0 || p + i >= count) return 0;
-                    loads[p + i] += 1;
+                    const long long at = (long long)(p + i) - misalign;
+                    if (at < 0 || at >= count) return 0;
+                    loads[at] += 1;
                 }
         }
+    return 1;
+}
+
+// One row [beg, end) of a pattern that ends with it, `warps` warps sharing it.  0: a load behind the pattern, or more iterations
+// than the row has chunks.
+extern "C" int table_row_at(int beg, int end, unsigned misalign, int warps, unsigned char *loads)
+{
+    const TableRow tr{beg + misalign, end + misalign, load_limit(end + misalign, 0, 1, end)};
+    for (int warp = 0; warp < warps; ++warp) {
+        int iterations = 0;
+        for (unsigned p0 = tr.first() + kMasksChunk * warp; p0 < tr.end; p0 += kMasksChunk * warps) {
+            if (++iterations > (end - beg) / (int)kMasksChunk + 2) return 0;
+            for (int lane = 0; lane < 32; ++lane) {
+                const unsigned p = p0 + kMasksRun * lane;
+                if (p >= tr.end) break;
+                for (unsigned i = 0; i < kMasksRun; ++i) {
+                    if (tr.has(p + i)) loads[p + i - tr.beg] += 1;
+                    else if (tr.wide(p) && p + i >= tr.end) return 0;
+                }
+            }
+        }
+    }
     return 1;
 }
 """
@@ -57,3 +80,14 @@ def test_the_table_pass_stays_inside_the_pattern(host, batch, last, slack, misal
             assert host.table_row(rp.ctypes.data_as(ctypes.c_void_p), row, ctypes.c_longlong(count + slack), batch, last, misalign,
                                   count if last else count + slack, loads.ctypes.data_as(ctypes.c_void_p)), (lens, row)
             assert (loads[rp[row]:rp[row + 1]] == 1).all()
+
+
+@pytest.mark.parametrize("warps", [1, 4])
+@pytest.mark.parametrize("length", [1, 31, 700, 2500])
+def test_the_table_pass_ends_at_the_largest_positions(host, length, warps):
+    """The last entry of a row may be number 2^31 - 2: steps past it must not wrap round."""
+    for end in (2 ** 31 - 1, 2 ** 31 - 2, 2 ** 31 - 260, 2 ** 31 - 1030):
+        for misalign in range(4):
+            loads = np.zeros(length, np.uint8)
+            assert host.table_row_at(end - length, end, misalign, warps, loads.ctypes.data_as(ctypes.c_void_p)), end
+            assert (loads == 1).all()
