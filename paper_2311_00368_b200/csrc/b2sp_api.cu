@@ -65,11 +65,11 @@ b2sp_status check_workspace(void *ws, size_t have, size_t need)
 b2sp_status bin_rows(int M, const int *row_ptr, const Workspace &w, cudaStream_t st, int *launches)
 {
     if (cudaMemsetAsync(w.count, 0, 512, st) != cudaSuccess) return B2SP_ERR_CUDA;
-    int blocks = (M + 255) / 256;
+    const unsigned blocks = ((unsigned)M + 255u) / 256u;
     bin_count_kernel<<<blocks, 256, 0, st>>>(M, row_ptr, w.count);
     {   // a programmatic dependent of the counting kernel (it waits for the counts where it needs them)
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)blocks);
+        cfg.gridDim = dim3(blocks);
         cfg.blockDim = dim3(256);
         cfg.stream = st;
         cudaLaunchAttribute attr[1];

@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "row_walk.h"
+
 namespace b2sp {
 
 constexpr int kRowWarps = 4;
@@ -71,8 +73,8 @@ __global__ void bin_count_kernel(int M, const int *__restrict__ row_ptr, int *__
     grid_release_dependents();
     if (threadIdx.x < kBuckets) h[threadIdx.x] = 0;
     __syncthreads();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < M) atomicAdd(&h[bucket_of(row_ptr[i + 1] - row_ptr[i])], 1);
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < (unsigned)M) atomicAdd(&h[bucket_of(row_ptr[i + 1] - row_ptr[i])], 1);
     __syncthreads();
     if (threadIdx.x < kBuckets && h[threadIdx.x]) atomicAdd(&count[threadIdx.x], h[threadIdx.x]);
 }
@@ -85,9 +87,9 @@ __global__ void bin_scatter_kernel(int M, const int *__restrict__ row_ptr,
     __shared__ int base[kBuckets];
     if (threadIdx.x < kBuckets) h[threadIdx.x] = 0;
     __syncthreads();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
     int b = 0, r = 0;
-    if (i < M) {
+    if (i < (unsigned)M) {
         b = bucket_of(row_ptr[i + 1] - row_ptr[i]);
         r = atomicAdd(&h[b], 1);
     }
@@ -100,7 +102,7 @@ __global__ void bin_scatter_kernel(int M, const int *__restrict__ row_ptr,
         base[mine] = h[mine] ? start + atomicAdd(&cursor[mine], h[mine]) : 0;
     }
     __syncthreads();
-    if (i < M) row_order[base[b] + r] = i;
+    if (i < (unsigned)M) row_order[base[b] + r] = (int)i;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -281,8 +283,8 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / G::LPN, sl = lane % G::LPN;
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
+    for (BlockRows br(blockIdx.x, nrows, gridDim.x); br.more(); br.advance()) {
+        const int row = row_order ? row_order[br.row] : (int)br.row;
         const int col0 = blockIdx.y * G::SLAB + sl * V;
         bool live[U];
         VecF<V> acc[U];
@@ -298,22 +300,23 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
         int k = 0;
         float s = 0.f;
         const int chunk = chunk_of(end - beg);
+        RowChunks rc(beg, end, warp, kRowWarps, chunk);
         {
-            int p = beg + warp * chunk + lane;
-            if (p < end) {
+            const unsigned p = rc.at + lane;
+            if (p < rc.end) {
                 k = __ldg(col_idx + p);
                 s = __ldg(values + p);
             }
         }
-        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
-            int pn = c + kRowWarps * chunk + lane;
+        for (; rc.more(); rc.advance()) {
+            const unsigned pn = rc.next(lane);
             int kn = 0;
             float sn = 0.f;
-            if (pn < end) {
+            if (pn < rc.end) {
                 kn = __ldg(col_idx + pn);
                 sn = __ldg(values + pn);
             }
-            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, min(chunk, end - c), Dcol, ldd, live, sub);
+            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, rc.count(), Dcol, ldd, live, sub);
             k = kn;
             s = sn;
         }
@@ -394,19 +397,19 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
+    for (BlockRows br(blockIdx.x, nrows, gridDim.x); br.more(); br.advance()) {
+        const int row = row_order ? row_order[br.row] : (int)br.row;
         const int beg = row_ptr[row], end = row_ptr[row + 1];
         VecF<V> areg[KU > 0 ? KU : 1];
         load_a_row<V, KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
         const int slot = (lane & 7) * 4 + (lane >> 3);  // entry of the chunk this lane ends up holding
         const int chunk = chunk_of(end - beg);
-        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
-            int p = c + lane;
-            int k = p < end ? __ldg(col_idx + p) : 0;
-            const int cnt = min(chunk, end - c);
+        for (RowChunks rc(beg, end, warp, kRowWarps, chunk); rc.more(); rc.advance()) {
+            const unsigned p = rc.at + lane;
+            int k = p < rc.end ? __ldg(col_idx + p) : 0;
+            const int cnt = rc.count();
             float dp = sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
-            int q = c + slot;
+            const unsigned q = rc.at + slot;
             if (slot < cnt) out_values[q] = s_values ? s_values[q] * dp : dp;
         }
         __syncthreads();   // shared memory is reused by the next row
@@ -424,11 +427,11 @@ sddmm_row_scalar_kernel(int Kd, const int *__restrict__ row_ptr, const int *__re
     if (gate_closed(gate)) return;
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
+    for (BlockRows br(blockIdx.x, nrows, gridDim.x); br.more(); br.advance()) {
+        const int row = row_order ? row_order[br.row] : (int)br.row;
         const int beg = row_ptr[row], end = row_ptr[row + 1];
         const DT *a = A + (int64_t)row * lda;
-        for (int p = beg + threadIdx.x; p < end; p += kRowThreads) {
+        for (unsigned p = beg + threadIdx.x; p < (unsigned)end; p += kRowThreads) {
             const DT *b = B + (int64_t)__ldg(col_idx + p) * ldb;
             float dp = 0.f;
             for (int l = 0; l < Kd; ++l) dp = fmaf(ldg1(a + l), ldg1(b + l), dp);
@@ -465,8 +468,8 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
     float *a_smem = reinterpret_cast<float *>(red + kRowWarps * U * G::LPN);  // Kd (KU == 0)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / G::LPN, sl = lane % G::LPN;
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
+    for (BlockRows br(blockIdx.x, nrows, gridDim.x); br.more(); br.advance()) {
+        const int row = row_order ? row_order[br.row] : (int)br.row;
         const int col0 = blockIdx.y * G::SLAB + sl * V;
         bool live[U];
         VecF<V> acc[U];
@@ -483,16 +486,17 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
         int k = 0;
         float sv = 1.f;
         const int chunk = chunk_of(end - beg);
+        RowChunks rc(beg, end, warp, kRowWarps, chunk);
         {
-            int p = beg + warp * chunk + lane, q = beg + warp * chunk + slot;
-            if (p < end) k = __ldg(col_idx + p);
-            if (s_values && q < end) sv = __ldg(s_values + q);
+            const unsigned p = rc.at + lane, q = rc.at + slot;
+            if (p < rc.end) k = __ldg(col_idx + p);
+            if (s_values && q < rc.end) sv = __ldg(s_values + q);
         }
-        for (int c = beg + warp * chunk; c < end; c += kRowWarps * chunk) {
-            int pn = c + kRowWarps * chunk + lane, qn = c + kRowWarps * chunk + slot;
-            int kn = pn < end ? __ldg(col_idx + pn) : 0;
-            float svn = (s_values && qn < end) ? __ldg(s_values + qn) : 1.f;
-            const int cnt = min(chunk, end - c);
+        for (; rc.more(); rc.advance()) {
+            const unsigned pn = rc.next(lane), qn = rc.next(slot);
+            int kn = pn < rc.end ? __ldg(col_idx + pn) : 0;
+            float svn = (s_values && qn < rc.end) ? __ldg(s_values + qn) : 1.f;
+            const int cnt = rc.count();
             float cv = sv * sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
             saxpy_chunk<V, U, SPLIT, true, DT>(acc, k, cv, cnt, Dcol, ldd, live, sub);
             k = kn;
@@ -523,23 +527,23 @@ fusedmm_row_scalar_kernel(int Kd, int N, const int *__restrict__ row_ptr,
     if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0;
     if (row_order) grid_wait_for_primary();   // launched behind the binning pass: its row order
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int rb = blockIdx.x; rb < nrows; rb += gridDim.x) {
-        const int row = row_order ? row_order[rb] : rb;
+    for (BlockRows br(blockIdx.x, nrows, gridDim.x); br.more(); br.advance()) {
+        const int row = row_order ? row_order[br.row] : (int)br.row;
         const int col0 = blockIdx.y * 128 + lane;
         float acc[4] = {0.f, 0.f, 0.f, 0.f};
         const int beg = row_ptr[row], end = row_ptr[row + 1];
         const DT *a = A + (int64_t)row * lda;
-        for (int c = beg + warp * 32; c < end; c += kRowWarps * 32) {
-            int p = c + lane;
+        for (RowChunks rc(beg, end, warp, kRowWarps, 32); rc.more(); rc.advance()) {
+            const unsigned p = rc.at + lane;
             int k = 0;
             float cv = 0.f;
-            if (p < end) {
+            if (p < rc.end) {
                 k = __ldg(col_idx + p);
                 const DT *b = B + (int64_t)k * ldb;
                 for (int l = 0; l < Kd; ++l) cv = fmaf(ldg1(a + l), ldg1(b + l), cv);
                 if (s_values) cv *= __ldg(s_values + p);
             }
-            int cnt = min(32, end - c);
+            const int cnt = rc.count();
             for (int j = 0; j < cnt; ++j) {
                 int kk = __shfl_sync(kFull, k, j);
                 float ss = __shfl_sync(kFull, cv, j);

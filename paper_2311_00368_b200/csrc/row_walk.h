@@ -36,4 +36,27 @@ struct TableRow {
     B2SP_HD bool has(unsigned p) const { return p >= beg && p < end; }
 };
 
+// ---- row kernels ---------------------------------------------------------------------------------
+// Rows and positions are unsigned here too: both may number 2^31 - 1, and a step past the last one still fits.
+// The rows of a block of a grid of `blocks`: block, block + blocks, ...
+struct BlockRows {
+    unsigned row, rows, step;
+    B2SP_HD BlockRows(unsigned block, unsigned rows_, unsigned blocks) : row(block), rows(rows_), step(blocks) {}
+    B2SP_HD bool more() const { return row < rows; }
+    B2SP_HD void advance() { row += step; }
+};
+
+// The chunks of a row [beg, end) that warp `warp` of `warps` takes: every warps-th one.
+struct RowChunks {
+    unsigned at, end, step, size;   // the chunk begins at `at`
+    B2SP_HD RowChunks(unsigned beg, unsigned end_, unsigned warp, unsigned warps, unsigned size_)
+        : at(beg + warp * size_), end(end_), step(warps * size_), size(size_)
+    {
+    }
+    B2SP_HD bool more() const { return at < end; }
+    B2SP_HD void advance() { at += step; }
+    B2SP_HD int count() const { return (int)(end - at < size ? end - at : size); }
+    B2SP_HD unsigned next(int i) const { return at + step + i; }   // entry i of the warp's next chunk (behind the row: not < end)
+};
+
 }  // namespace b2sp

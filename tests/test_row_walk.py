@@ -54,6 +54,30 @@ extern "C" int table_row_at(int beg, int end, unsigned misalign, int warps, unsi
     }
     return 1;
 }
+
+// A row kernel's walk over a row [beg, end): every entry is taken once, and a prefetch that says it is inside the row is.
+extern "C" int row_chunks(int beg, int end, int warps, int size, unsigned char *taken)
+{
+    for (int warp = 0; warp < warps; ++warp) {
+        int iterations = 0;
+        for (RowChunks r(beg, end, warp, warps, size); r.more(); r.advance()) {
+            if (++iterations > (end - beg) / size + 1) return 0;
+            for (int i = 0; i < (int)r.count(); ++i) taken[(long long)r.at + i - beg] += 1;
+            for (int lane = 0; lane < 32; ++lane)
+                if (r.next(lane) < r.end && ((long long)r.next(lane) < beg || (long long)r.next(lane) >= end)) return 0;
+        }
+    }
+    return 1;
+}
+
+extern "C" int block_rows(int block, int rows, int blocks)   // rows that a block walks; -1: one that does not exist
+{
+    int n = 0;
+    for (BlockRows b(block, rows, blocks); b.more(); b.advance()) {
+        if ((long long)b.row < 0 || (long long)b.row >= rows || ++n > 4) return -1;
+    }
+    return n;
+}
 """
 
 
@@ -91,3 +115,18 @@ def test_the_table_pass_ends_at_the_largest_positions(host, length, warps):
             loads = np.zeros(length, np.uint8)
             assert host.table_row_at(end - length, end, misalign, warps, loads.ctypes.data_as(ctypes.c_void_p)), end
             assert (loads == 1).all()
+
+
+@pytest.mark.parametrize("size", [4, 12, 16, 32])
+@pytest.mark.parametrize("length", [1, 16, 33, 64, 65, 129, 700])
+def test_the_row_kernels_take_every_entry_once(host, length, size):
+    for end in (length, 1000 + length, 2 ** 31 - 1, 2 ** 31 - 2, 2 ** 31 - 100, 2 ** 31 - 160):
+        taken = np.zeros(length, np.uint8)
+        assert host.row_chunks(end - length, end, 4, size, taken.ctypes.data_as(ctypes.c_void_p)), end
+        assert (taken == 1).all()
+
+
+@pytest.mark.parametrize("rows,blocks,block,want", [(10, 10, 9, 1), (10, 4, 1, 3), (2 ** 31 - 1, 2 ** 31 - 1, 2 ** 31 - 2, 1),
+                                                    (2 ** 30 + 5, 2 ** 30 + 5, 2 ** 30 + 4, 1), (2 ** 30, 2 ** 30, 7, 1)])
+def test_a_block_walks_its_rows(host, rows, blocks, block, want):
+    assert host.block_rows(block, rows, blocks) == want
