@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "row_kernels.cuh"
 #include "tile_dispatch.h"
@@ -113,14 +114,14 @@ inline unsigned gated_blocks(unsigned rows, int *gate, unsigned nbatch = 1)
     return gate && rows > cap ? cap : rows;
 }
 
-template <int V, int U, int SPLIT, typename DT>
+template <int V, int U, int SPLIT, bool SHORT, typename DT>
 void launch_spmm(dim3 grid, cudaStream_t st, int N, const int *row_ptr, const int *col_idx,
                  const float *values, const DT *D, int64_t ldd, float *O, int64_t ldo,
                  const int *order, int *gate, int *clear)
 {
     const int nrows = (int)grid.x;
     grid.x = gated_blocks(grid.x, gate);
-    launch_row(spmm_row_kernel<V, U, SPLIT, DT>, grid, 0, st, gate != nullptr || order != nullptr, N, row_ptr, col_idx, values, D, ldd, O, ldo, order,
+    launch_row(spmm_row_kernel<V, U, SPLIT, SHORT, DT>, grid, 0, st, gate != nullptr || order != nullptr, N, row_ptr, col_idx, values, D, ldd, O, ldo, order,
                gate, nrows, clear);
 }
 
@@ -156,7 +157,31 @@ inline int pick_ku(int Kd, int V)
     return V == 4 && Kd <= 256 ? 8 : 0;
 }
 
-template <int V, int KU, typename DT>
+// Where the form of a row kernel for long rows exists (see row_kernels.cuh), and up to which average row length the form for short
+// rows is chosen beside it.  Measured over 40 to 1600 entries a row (4096 rows), us of the short and the long form; every width
+// that is missing here is served better, or as well, by the form for short rows over the whole range.
+template <int V, int U, int SPLIT> constexpr bool spmm_has_long() { return V == 4 && (SPLIT == 2 || U >= 2); }
+template <int V, int KU, typename DT> constexpr bool sddmm_has_long() { return V == 4 && (KU == 2 || (KU == 8 && sizeof(DT) == 2)); }
+template <int V, int KU, int U, int SPLIT, typename DT> constexpr bool fused_has_long()
+{
+    return V == 4 && (KU == 2 ? U <= 2 : KU == 4 ? SPLIT == 1 : KU == 8 && sizeof(DT) == 4 && U == 2);
+}
+inline bool short_rows(long long nnz, int M, int entries) { return nnz <= (long long)entries * M; }
+// x 64: 130 entries 15.0 / 15.3, 300 27.3 / 26.0; power law 8192 x 8192 at 10% 156 / 134.  x 256: 130 entries 31.9 / 33.3, 205
+// 46.3 / 44.8, 1600 314 / 300, but with less than a wave of rows the loads in flight are worth more (300 x 4096, 614 entries: 26.6 /
+// 30.2).  x 512: 40 entries 24.0 / 32.7, 80 39.7 / 39.8; bf16 60 entries 30.0 / 29.0, 205 71.8 / 67.9.
+template <int U, int SPLIT> inline bool spmm_short(long long nnz, int M)
+{
+    return short_rows(nnz, M, U == 4 ? 72 : 144) || (U == 2 && M < 148 * 10);
+}
+// Kd = 64: 100 entries 12.4 / 12.7, 130 15.5 / 15.1; bf16 Kd = 256: 100 35.8 / 36.8, 205 64.0 / 62.5.
+inline bool sddmm_short(long long nnz, int M) { return short_rows(nnz, M, 128); }
+// Kd = N = 64: 130 entries 27.2 / 30.3, 205 38.2 / 37.2, 1600 224 / 207; Kd = N = 128: 60 28.4 / 35.5, 100 36.8 / 36.5, 205 63.8 / 58.8,
+// 1600 382 / 333 (1024 x 1024 at 20%: 25.8 / 18.6); Kd = 128, N = 256: 130 54.5 / 58.5, 205 77.5 / 75.0.  Rows of 128 bytes or less:
+// Kd = N = 32: 60 13.5 / 14.8, 80 15.6 / 15.2, 450 52.8 / 48.6; bf16 Kd = N = 64: 60 17.4 / 17.8, 100 20.5 / 19.6, 900 128 / 113.
+template <typename DT> inline bool fused_short(long long nnz, int M, int N) { return short_rows(nnz, M, N * (int)sizeof(DT) <= 128 ? 72 : 144); }
+
+template <int V, int KU, bool SHORT, typename DT>
 void launch_sddmm(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const int *col_idx,
                   const float *sv, const DT *A, int64_t lda, const DT *B, int64_t ldb,
                   float *out, const int *order, int *gate, int *clear)
@@ -164,11 +189,11 @@ void launch_sddmm(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const 
     size_t smem = KU == 0 ? sizeof(float) * (size_t)((Kd + 3) & ~3) : 0;
     const int nrows = (int)grid.x;
     grid.x = gated_blocks(grid.x, gate);
-    launch_row(sddmm_row_kernel<V, KU, DT>, grid, smem, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, sv, A, lda, B, ldb, out, order,
+    launch_row(sddmm_row_kernel<V, KU, SHORT, DT>, grid, smem, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, sv, A, lda, B, ldb, out, order,
                gate, nrows, clear);
 }
 
-template <int V, int KU, int U, int SPLIT, typename DT>
+template <int V, int KU, int U, int SPLIT, bool SHORT, typename DT>
 b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *row_ptr,
                          const int *col_idx, const float *sv, const DT *A, int64_t lda,
                          const DT *B, int64_t ldb, const DT *D, int64_t ldd, float *O,
@@ -177,8 +202,8 @@ b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *r
     size_t smem = sizeof(VecF<V>) * kRowWarps * U * (32 / SPLIT) +
                   (KU == 0 ? sizeof(float) * (size_t)((Kd + 3) & ~3) : 0);
     const bool batched = grid.z > 1;
-    auto kern_b = fusedmm_row_kernel<V, KU, U, SPLIT, true, DT>;
-    auto kern_1 = fusedmm_row_kernel<V, KU, U, SPLIT, false, DT>;
+    auto kern_b = fusedmm_row_kernel<V, KU, U, SPLIT, SHORT, true, DT>;
+    auto kern_1 = fusedmm_row_kernel<V, KU, U, SPLIT, SHORT, false, DT>;
     if (smem > 48 * 1024) {
         if (smem > 200 * 1024) return B2SP_ERR_UNSUPPORTED;
         if (cudaFuncSetAttribute(batched ? reinterpret_cast<const void *>(kern_b) : reinterpret_cast<const void *>(kern_1),
@@ -196,43 +221,39 @@ b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *r
     return B2SP_OK;
 }
 
-template <int V, int KU, typename DT>
-b2sp_status dispatch_fused_geom(const Geom &g, dim3 grid, cudaStream_t st, int Kd, int N,
-                                const int *row_ptr, const int *col_idx, const float *sv,
-                                const DT *A, int64_t lda, const DT *B, int64_t ldb,
-                                const DT *D, int64_t ldd, float *O, int64_t ldo,
-                                const int *order, int *gate, int *clear, const RowBatch &rb)
+template <int V, int KU, int U, int SPLIT, typename DT, class... Args>
+b2sp_status launch_fused_form(bool is_short, Args... args)
 {
-#define B2SP_F(U_, S_) \
-    return launch_fused<V, KU, U_, S_, DT>(grid, st, Kd, N, row_ptr, col_idx, sv, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
-    if constexpr (V == 4) {
-        if (g.SPLIT == 4) B2SP_F(1, 4);
+    if constexpr (fused_has_long<V, KU, U, SPLIT, DT>()) {
+        if (!is_short) return launch_fused<V, KU, U, SPLIT, false, DT>(args...);
     }
-    if (g.SPLIT == 2) B2SP_F(1, 2);
-    if (g.U == 1) B2SP_F(1, 1);
-    if constexpr (V == 2) B2SP_F(2, 1);
-    else if (g.U == 2) B2SP_F(2, 1);
-    else B2SP_F(4, 1);
-#undef B2SP_F
+    return launch_fused<V, KU, U, SPLIT, true, DT>(args...);
 }
 
-template <int V, typename DT>
-b2sp_status dispatch_fused_ku(const Geom &g, dim3 grid, cudaStream_t st, int Kd, int N,
-                              const int *row_ptr, const int *col_idx, const float *sv,
-                              const DT *A, int64_t lda, const DT *B, int64_t ldb,
-                              const DT *D, int64_t ldd, float *O, int64_t ldo,
-                              const int *order, int *gate, int *clear, const RowBatch &rb)
+template <int V, int KU, typename DT, class... Args>
+b2sp_status dispatch_fused_geom(const Geom &g, Args... args)
+{
+    if constexpr (V == 4) {
+        if (g.SPLIT == 4) return launch_fused_form<V, KU, 1, 4, DT>(args...);
+    }
+    if (g.SPLIT == 2) return launch_fused_form<V, KU, 1, 2, DT>(args...);
+    if (g.U == 1) return launch_fused_form<V, KU, 1, 1, DT>(args...);
+    if constexpr (V == 2) return launch_fused_form<V, KU, 2, 1, DT>(args...);
+    else if (g.U == 2) return launch_fused_form<V, KU, 2, 1, DT>(args...);
+    else return launch_fused_form<V, KU, 4, 1, DT>(args...);
+}
+
+// `args`: is_short and launch_fused's.
+template <int V, typename DT, class... Args>
+b2sp_status dispatch_fused_ku(const Geom &g, int Kd, Args... args)
 {
     const int ku = pick_ku(Kd, V);
-#define B2SP_F(KU_) \
-    return dispatch_fused_geom<V, KU_, DT>(g, grid, st, Kd, N, row_ptr, col_idx, sv, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
-    if (ku == 8 / V) B2SP_F(8 / V);
-    if (ku == 16 / V) B2SP_F(16 / V);
+    if (ku == 8 / V) return dispatch_fused_geom<V, 8 / V, DT>(g, args...);
+    if (ku == 16 / V) return dispatch_fused_geom<V, 16 / V, DT>(g, args...);
     if constexpr (V == 4) {
-        if (ku == 8) B2SP_F(8);
+        if (ku == 8) return dispatch_fused_geom<V, 8, DT>(g, args...);
     }
-    B2SP_F(0);
-#undef B2SP_F
+    return dispatch_fused_geom<V, 0, DT>(g, args...);
 }
 
 b2sp_status zero_rows(float *O, int64_t ldo, int M, int N, cudaStream_t st)
@@ -331,14 +352,24 @@ static int auto_row_algo(int M) { return M <= 4096 ? B2SP_ALGO_ROW_NAT : B2SP_AL
 
 // Enqueues the row-family SPMM.  `gate` != NULL makes it a device-side fallback.
 template <typename DT>
-static b2sp_status spmm_rows(int M, int N, const int *row_ptr, const int *col_idx, const float *values,
+static b2sp_status spmm_rows(int M, int N, long long nnz, const int *row_ptr, const int *col_idx, const float *values,
                              const DT *D, long long ldd, float *O, long long ldo, const int *order,
                              int *gate, int *clear, cudaStream_t st)
 {
     const int V = std::min(vec_width(D, N, ldd), vec_width(O, N, ldo));
     const Geom g = pick_geom(N, V);
     dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab));
-#define B2SP_S(V_, U_, S_) launch_spmm<V_, U_, S_, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear)
+    auto launch = [&](auto v, auto u, auto split) {
+        constexpr int V_ = decltype(v)::value, U_ = decltype(u)::value, S_ = decltype(split)::value;
+        if constexpr (spmm_has_long<V_, U_, S_>()) {
+            if (!spmm_short<U_, S_>(nnz, M)) {
+                launch_spmm<V_, U_, S_, false, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
+                return;
+            }
+        }
+        launch_spmm<V_, U_, S_, true, DT>(grid, st, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, gate, clear);
+    };
+#define B2SP_S(V_, U_, S_) launch(std::integral_constant<int, V_>(), std::integral_constant<int, U_>(), std::integral_constant<int, S_>())
     if (V == 4) {
         if (g.SPLIT == 4) B2SP_S(4, 1, 4);
         else if (g.SPLIT == 2) B2SP_S(4, 1, 2);
@@ -393,7 +424,7 @@ static b2sp_status spmm_impl(int M, int K, int N, long long nnz, const int *row_
         if (rc != B2SP_OK) return rc;
         // device-side fallback: runs only if the pre-pass found rows that are not strictly sorted
         int *gate = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsTileFlagsOffset);
-        rc = spmm_rows(M, N, row_ptr, col_idx, values, D, ldd, O, ldo, nullptr, gate, nullptr, st);
+        rc = spmm_rows(M, N, nnz, row_ptr, col_idx, values, D, ldd, O, ldo, nullptr, gate, nullptr, st);
         g_last_launches[B2SP_OP_SPMM] = launches + 1;
         return rc;
     }
@@ -406,36 +437,43 @@ static b2sp_status spmm_impl(int M, int K, int N, long long nnz, const int *row_
     } else {   // no binning pass: the row kernel itself resets the status word
         clear = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsStatusOffset);
     }
-    rc = spmm_rows(M, N, row_ptr, col_idx, values, D, ldd, O, ldo, order, nullptr, clear, st);
+    rc = spmm_rows(M, N, nnz, row_ptr, col_idx, values, D, ldd, O, ldo, order, nullptr, clear, st);
     g_last_launches[B2SP_OP_SPMM] = launches + 1;
     return rc;
 }
 
 // Picks the SDDMM kernel that holds A_i for this Kd.
 template <int V, typename DT>
-static b2sp_status dispatch_sddmm_ku(dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const int *col_idx, const float *s_values,
+static b2sp_status dispatch_sddmm_ku(bool is_short, dim3 grid, cudaStream_t st, int Kd, const int *row_ptr, const int *col_idx, const float *s_values,
                                      const DT *A, long long lda, const DT *B, long long ldb, float *out_values, const int *order,
                                      int *gate, int *clear)
 {
     const int ku = pick_ku(Kd, V);
-#define B2SP_C(KU_) launch_sddmm<V, KU_, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
-    if (ku == 8 / V) { B2SP_C(8 / V); return B2SP_OK; }
-    if (ku == 16 / V) { B2SP_C(16 / V); return B2SP_OK; }
+#define B2SP_C(KU_, SHORT_) launch_sddmm<V, KU_, SHORT_, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+    auto launch = [&](auto groups) {
+        constexpr int KU = decltype(groups)::value;
+        if constexpr (sddmm_has_long<V, KU, DT>()) {
+            if (!is_short) { B2SP_C(KU, false); return; }
+        }
+        B2SP_C(KU, true);
+    };
+    if (ku == 8 / V) { launch(std::integral_constant<int, 8 / V>()); return B2SP_OK; }
+    if (ku == 16 / V) { launch(std::integral_constant<int, 16 / V>()); return B2SP_OK; }
     if constexpr (V == 4) {
-        if (ku == 8) { B2SP_C(8); return B2SP_OK; }
+        if (ku == 8) { launch(std::integral_constant<int, 8>()); return B2SP_OK; }
     }
     const size_t smem = sizeof(float) * (size_t)((Kd + 3) & ~3);
     if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(sddmm_row_kernel<V, 0, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(sddmm_row_kernel<V, 0, true, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return B2SP_ERR_CUDA;
-    B2SP_C(0);
+    B2SP_C(0, true);
 #undef B2SP_C
     return B2SP_OK;
 }
 
 // Enqueues the row-family SDDMM.  `gate` != NULL makes it a device-side fallback.
 template <typename DT>
-static b2sp_status sddmm_rows(int M, int Kd, const int *row_ptr, const int *col_idx, const float *s_values,
+static b2sp_status sddmm_rows(int M, int Kd, long long nnz, const int *row_ptr, const int *col_idx, const float *s_values,
                               const DT *A, long long lda, const DT *B, long long ldb,
                               float *out_values, const int *order, int *gate, int *clear, cudaStream_t st)
 {
@@ -448,9 +486,9 @@ static b2sp_status sddmm_rows(int M, int Kd, const int *row_ptr, const int *col_
     }
     const int V = std::min(vec_width(A, Kd, lda), vec_width(B, Kd, ldb));
     const b2sp_status rc =
-        V == 4 ? dispatch_sddmm_ku<4, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
-        : V == 2 ? dispatch_sddmm_ku<2, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
-                 : dispatch_sddmm_ku<1, DT>(grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear);
+        V == 4 ? dispatch_sddmm_ku<4, DT>(sddmm_short(nnz, M), grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+        : V == 2 ? dispatch_sddmm_ku<2, DT>(sddmm_short(nnz, M), grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
+                 : dispatch_sddmm_ku<1, DT>(sddmm_short(nnz, M), grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear);
     if (rc != B2SP_OK) return rc;
     return check_launch();
 }
@@ -492,7 +530,7 @@ static b2sp_status sddmm_impl(int M, int K, int Kd, long long nnz, const int *ro
                         out_values, 0, workspace, st, &launches, false, BatchDesc(), dense_dtype<DT>());
         if (rc != B2SP_OK) return rc;
         int *gate = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsTileFlagsOffset);
-        rc = sddmm_rows(M, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, nullptr, gate, nullptr, st);
+        rc = sddmm_rows(M, Kd, nnz, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, nullptr, gate, nullptr, st);
         g_last_launches[B2SP_OP_SDDMM] = launches + 1;
         return rc;
     }
@@ -505,14 +543,14 @@ static b2sp_status sddmm_impl(int M, int K, int Kd, long long nnz, const int *ro
     } else {   // no binning pass: the row kernel itself resets the status word
         clear = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsStatusOffset);
     }
-    rc = sddmm_rows(M, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, nullptr, clear, st);
+    rc = sddmm_rows(M, Kd, nnz, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, nullptr, clear, st);
     g_last_launches[B2SP_OP_SDDMM] = launches + 1;
     return rc;
 }
 
 // Enqueues the row-family FusedMM.  `gate` != NULL makes it a device-side fallback.
 template <typename DT>
-static b2sp_status fused_rows(int M, int Kd, int N, const int *row_ptr, const int *col_idx,
+static b2sp_status fused_rows(int M, int Kd, int N, long long nnz, const int *row_ptr, const int *col_idx,
                               const float *s_values, const DT *A, long long lda, const DT *B,
                               long long ldb, const DT *D, long long ldd, float *O, long long ldo,
                               const int *order, int *gate, int *clear, cudaStream_t st,
@@ -528,9 +566,10 @@ static b2sp_status fused_rows(int M, int Kd, int N, const int *row_ptr, const in
     const int V = std::min({vec_width(A, Kd, lda, rb.A), vec_width(B, Kd, ldb, rb.B), vec_width(D, N, ldd, rb.D), vec_width(O, N, ldo, rb.O)});
     const Geom g = pick_geom(N, V);
     dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab), (unsigned)nbatch);
-    rc = V == 4 ? dispatch_fused_ku<4, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
-         : V == 2 ? dispatch_fused_ku<2, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
-                  : dispatch_fused_ku<1, DT>(g, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb);
+    const bool is_short = fused_short<DT>(nnz, M, N);
+    rc = V == 4 ? dispatch_fused_ku<4, DT>(g, Kd, is_short, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+         : V == 2 ? dispatch_fused_ku<2, DT>(g, Kd, is_short, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb)
+                  : dispatch_fused_ku<1, DT>(g, Kd, is_short, grid, st, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, gate, clear, rb);
     if (rc != B2SP_OK) return rc;
     return check_launch();
 }
@@ -582,7 +621,7 @@ static b2sp_status fusedmm_impl(int M, int K, int Kd, int N, long long nnz, cons
         }
         if (rc != B2SP_OK) return rc;
         int *gate = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsTileFlagsOffset);
-        rc = fused_rows(M, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, gate, nullptr, st);
+        rc = fused_rows(M, Kd, N, nnz, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, gate, nullptr, st);
         g_last_launches[B2SP_OP_FUSEDMM] = launches + 1;
         return rc;
     }
@@ -595,7 +634,7 @@ static b2sp_status fusedmm_impl(int M, int K, int Kd, int N, long long nnz, cons
     } else {   // no binning pass: the row kernel itself resets the status word
         clear = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsStatusOffset);
     }
-    rc = fused_rows(M, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, nullptr, clear, st);
+    rc = fused_rows(M, Kd, N, nnz, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, order, nullptr, clear, st);
     g_last_launches[B2SP_OP_FUSEDMM] = launches + 1;
     return rc;
 }
@@ -745,13 +784,13 @@ static b2sp_status fusedmm_batched_impl(int batch, int M, int K, int Kd, int N, 
                         O, ldo, workspace, st, &launches, false, bd, dense_dtype<DT>());
         if (rc != B2SP_OK) return rc;
         int *gate = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsTileFlagsOffset);
-        rc = fused_rows(M, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, gate, nullptr, st,
+        rc = fused_rows(M, Kd, N, nnz_stride, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, gate, nullptr, st,
                         batch, rb);
         g_last_launches[B2SP_OP_FUSEDMM] = launches + 1;
         return rc;
     }
     int *clear = reinterpret_cast<int *>(static_cast<char *>(workspace) + kWsStatusOffset);
-    rc = fused_rows(M, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, nullptr, clear, st,
+    rc = fused_rows(M, Kd, N, nnz_stride, row_ptr, col_idx, s_values, A, lda, B, ldb, D, ldd, O, ldo, nullptr, nullptr, clear, st,
                     batch, rb);
     g_last_launches[B2SP_OP_FUSEDMM] = 1;
     return rc;

@@ -174,16 +174,21 @@ struct SweepGeom {
     static constexpr int SLAB = LPN * V * U;
 };
 
+// Two forms of the row kernels.  Short rows are cut into a chunk for each warp, and their partial chunks, which is all they
+// have, keep several entries' loads in flight.  That takes registers and a chunk length known at run time only, which long rows
+// pay for and have no use for: their form has chunks of 32 and the plainest loops for what is left of a row.  Where both are
+// instantiated the host chooses by the average row length (short_rows in b2sp_api.cu).
+
 // One chunk (up to 32 entries, lane l holds entry l: column k, scalar s) of the Alg. 2 SAXPY
 // sweep.  SRC(j) gives the lane that holds entry j's scalar.
-template <int V, int U, int SPLIT, bool PERMUTED, typename DT>
+template <int V, int U, int SPLIT, bool PERMUTED, bool SHORT, typename DT>
 __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, int cnt,
                                             const DT *__restrict__ Dcol, int64_t ldd,
                                             bool (&live)[U], int sub)
 {
     constexpr int LPN = 32 / SPLIT;
+    constexpr int STEPS = 32 / SPLIT;
     if (cnt == 32) {
-        constexpr int STEPS = 32 / SPLIT;
 #pragma unroll 8
         for (int jj = 0; jj < STEPS; ++jj) {
             int j = jj * SPLIT + sub;
@@ -195,12 +200,13 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
             for (int u = 0; u < U; ++u)
                 if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
         }
-    } else {
+    } else if constexpr (SHORT) {
         // Entries whose loads are in flight together.  It is a matter of registers, which the full chunks then miss, and was
         // measured: single or pair elements four (two: 1501 x 2903 x 71 spmm 24.8 -> 27.5 us); SPMM with whole warps two (one:
-        // 8192 x 8192 at 10% x 256 385 -> 514 us, x 128 248 -> 298 us); FusedMM and sub-warps one (two: 4096 x 4096 at 20% x 64
-        // spmm 69 -> 74 us, 8192 x 8192 at 5%, Kd = N = 32, fusedmm 90 -> 97 us).
-        constexpr int BATCH = V < 4 ? 4 : !PERMUTED && SPLIT == 1 ? 2 : 1;
+        // power law 8192 x 8192 at 10% x 256 382 -> 442 us), but one with four groups per lane (two: 77 registers instead of 62,
+        // 1024 x 1024 at 25% x 512 29.5 -> 38.5 us, 8192 x 8192 at 30% 1.68 -> 1.74 ms); FusedMM and sub-warps one (two: power law
+        // 8192 x 8192 at 10% x 64 spmm 156 -> 205 us, 8192 x 8192 at 5%, Kd = N = 32, fusedmm 90 -> 97 us).
+        constexpr int BATCH = V < 4 ? 4 : !PERMUTED && SPLIT == 1 && U < 4 ? 2 : 1;
         for (int jj = 0; jj * SPLIT < cnt; jj += BATCH) {
             VecF<V> d[BATCH][U];
             float ss[BATCH];
@@ -221,14 +227,29 @@ __device__ __forceinline__ void saxpy_chunk(VecF<V> (&acc)[U], int k, float s, i
                     for (int u = 0; u < U; ++u) fma_v<V>(acc[u], ss[i], d[i][u]);
                 }
         }
+    } else {
+        for (int jj = 0; jj < STEPS; ++jj) {
+            const int j = jj * SPLIT + sub;
+            const int src = PERMUTED ? ((j & 3) * 8 + (j >> 2)) : j;
+            const int kk = __shfl_sync(kFull, k, j);
+            const float ss = __shfl_sync(kFull, s, src);
+            if (j < cnt) {
+                const DT *d = Dcol + (int64_t)kk * ldd;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (live[u]) fma_v<V>(acc[u], ss, ldgv<V>(d + u * LPN * V));
+            }
+        }
     }
 }
 
-// Entries of a row that a warp takes at a time: 32, or a quarter of a row of 64 or fewer (a multiple of four, the groups of
-// sddmm_chunk), so that all four warps have a part of it: a row of 25 entries was one warp's serial chain while three idled
-// (256 x 256 at 10%, Kd = N = 64, fusedmm: 7.1 -> 4.0 us; 4096 x 512 at 5%, Kd = 100, N = 250: 83 -> 32 us).  With the line at
-// 128 entries, rows of 102 lost their full chunks' eight loads in flight (3072 x 1024 x 32 spmm 7.1 -> 7.5 us).
-__device__ __forceinline__ int chunk_of(int len) { return len > 64 ? 32 : ((len + 4 * kRowWarps - 1) / (4 * kRowWarps)) * 4; }
+// Entries of a row that a warp takes at a time: 32; in the form for short rows a quarter of a row of 64 or fewer, rounded up to
+// groups of four (those of sddmm_chunk), so that the four warps share it: a row of 25 entries was one warp's serial chain while
+// three idled (256 x 256 at 10%, Kd = N = 64, fusedmm: 7.1 -> 4.0 us; 4096 x 512 at 5%, Kd = 100, N = 250: 66 -> 32 us).  Between
+// 65 and about 110 entries the warps' parts are uneven (65: 32, 32, 1 and 0); with the line at 128 instead, rows of 102 lost their
+// full chunks' eight loads in flight (3072 x 1024 x 32 spmm 7.1 -> 7.5 us).
+template <bool SHORT>
+__device__ __forceinline__ int chunk_of(int len) { return !SHORT || len > 64 ? 32 : ((len + 4 * kRowWarps - 1) / (4 * kRowWarps)) * 4; }
 
 // Combine the sub-warps of a warp, then the warps of the CTA (fixed order), and store the row.
 template <int V, int U, int SPLIT>
@@ -269,7 +290,7 @@ __device__ __forceinline__ void reduce_and_store_row(VecF<V> (&acc)[U], VecF<V> 
 // ------------------------------------------------------------------------------------------
 // SPMM  (Alg. 2; N, ldd, ldo multiples of V, D and O aligned to V elements)
 // ------------------------------------------------------------------------------------------
-template <int V, int U, int SPLIT, typename DT>
+template <int V, int U, int SPLIT, bool SHORT, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                 const float *__restrict__ values, const DT *__restrict__ D, int64_t ldd,
@@ -299,7 +320,7 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
         // (the role of the paper's prefetch of the next ja/avalues block)
         int k = 0;
         float s = 0.f;
-        const int chunk = chunk_of(end - beg);
+        const int chunk = chunk_of<SHORT>(end - beg);
         RowChunks rc(beg, end, warp, kRowWarps, chunk);
         {
             const unsigned p = rc.at + lane;
@@ -316,7 +337,7 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
                 kn = __ldg(col_idx + pn);
                 sn = __ldg(values + pn);
             }
-            saxpy_chunk<V, U, SPLIT, false, DT>(acc, k, s, rc.count(), Dcol, ldd, live, sub);
+            saxpy_chunk<V, U, SPLIT, false, SHORT, DT>(acc, k, s, rc.count(), Dcol, ldd, live, sub);
             k = kn;
             s = sn;
         }
@@ -334,7 +355,7 @@ spmm_row_kernel(int N, const int *__restrict__ row_ptr, const int *__restrict__ 
 // group g takes entries 4r + g (r = 0..7); after the 3-step butterfly every lane of the
 // group has the sum and lane t keeps round t's, so lane 8g + t ends up holding entry 4t + g.
 // ------------------------------------------------------------------------------------------
-template <int V, int KU, typename DT>
+template <int V, int KU, bool SHORT, bool FUSED, typename DT>
 __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU : 1],
                                              const float *__restrict__ a_smem, int Kd, int k,
                                              const DT *__restrict__ B, int64_t ldb, int lane, int cnt)
@@ -358,7 +379,18 @@ __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU :
         part += __shfl_xor_sync(kFull, part, 4);
         if (r == t) mine = part;
     };
-    if (cnt == 32) {
+    if constexpr (!SHORT) {   // (rounds behind the end of the row read row 0 of B)
+#pragma unroll 4
+        for (int r = 0; r < 8; ++r) round(r);
+    } else if constexpr (!FUSED && KU == 8 && sizeof(DT) == 4) {
+        // four rounds at a time and no second loop: with it 128 < Kd <= 256 took longer than with eight rounds for every chunk,
+        // this way less (4096 x 1024 at 20%, Kd = 256: 73.0, 68.2 and 59.9 us; rows of 40 entries: 19.1, 34.9 and 20.9)
+#pragma unroll 1
+        for (int r0 = 0; 4 * r0 < cnt; r0 += 4) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r) round(r0 + r);
+        }
+    } else if (cnt == 32) {
 #pragma unroll 4
         for (int r = 0; r < 8; ++r) round(r);
     } else {   // (one loop for both, its length known only at run time, cost full chunks a quarter of their speed)
@@ -384,7 +416,7 @@ __device__ __forceinline__ void load_a_row(VecF<V> (&areg)[KU > 0 ? KU : 1], flo
     }
 }
 
-template <int V, int KU, typename DT>
+template <int V, int KU, bool SHORT, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                  const float *s_values, const DT *__restrict__ A, int64_t lda,
@@ -403,12 +435,12 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
         VecF<V> areg[KU > 0 ? KU : 1];
         load_a_row<V, KU, DT>(areg, a_smem, A + (int64_t)row * lda, Kd, lane);
         const int slot = (lane & 7) * 4 + (lane >> 3);  // entry of the chunk this lane ends up holding
-        const int chunk = chunk_of(end - beg);
+        const int chunk = chunk_of<SHORT>(end - beg);
         for (RowChunks rc(beg, end, warp, kRowWarps, chunk); rc.more(); rc.advance()) {
             const unsigned p = rc.at + lane;
             int k = p < rc.end ? __ldg(col_idx + p) : 0;
             const int cnt = rc.count();
-            float dp = sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
+            float dp = sddmm_chunk<V, KU, SHORT, false, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
             const unsigned q = rc.at + slot;
             if (slot < cnt) out_values[q] = s_values ? s_values[q] * dp : dp;
         }
@@ -445,7 +477,7 @@ sddmm_row_scalar_kernel(int Kd, const int *__restrict__ row_ptr, const int *__re
 // FusedMM  (Alg. 3): per chunk, the SDDMM values stay in registers (one per lane) and are the
 // scalars of the SAXPY sweep over the same staged column indices; C never reaches memory.
 // ------------------------------------------------------------------------------------------
-template <int V, int KU, int U, int SPLIT, bool BATCHED, typename DT>
+template <int V, int KU, int U, int SPLIT, bool SHORT, bool BATCHED, typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,
                    const float *__restrict__ s_values, const DT *__restrict__ A, int64_t lda,
@@ -485,7 +517,7 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
         const DT *Dcol = D + col0;
         int k = 0;
         float sv = 1.f;
-        const int chunk = chunk_of(end - beg);
+        const int chunk = chunk_of<SHORT>(end - beg);
         RowChunks rc(beg, end, warp, kRowWarps, chunk);
         {
             const unsigned p = rc.at + lane, q = rc.at + slot;
@@ -494,11 +526,15 @@ fusedmm_row_kernel(int Kd, int N, const int *__restrict__ row_ptr, const int *__
         }
         for (; rc.more(); rc.advance()) {
             const unsigned pn = rc.next(lane), qn = rc.next(slot);
-            int kn = pn < rc.end ? __ldg(col_idx + pn) : 0;
-            float svn = (s_values && qn < rc.end) ? __ldg(s_values + qn) : 1.f;
+            // (the same test in two ways: with the first the long form for 64 < Kd <= 128 spilled a register on bfloat16, 102 -> 116 us
+            // at 450 entries a row; with the second it did for Kd = N = 32, 48.6 -> 51.3 us)
+            constexpr bool BY_COUNT = !SHORT && KU >= 4;
+            const bool has_p = BY_COUNT ? lane < rc.behind() : pn < rc.end, has_q = BY_COUNT ? slot < rc.behind() : qn < rc.end;
+            int kn = has_p ? __ldg(col_idx + pn) : 0;
+            float svn = (s_values && has_q) ? __ldg(s_values + qn) : 1.f;
             const int cnt = rc.count();
-            float cv = sv * sddmm_chunk<V, KU, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
-            saxpy_chunk<V, U, SPLIT, true, DT>(acc, k, cv, cnt, Dcol, ldd, live, sub);
+            float cv = sv * sddmm_chunk<V, KU, SHORT, true, DT>(areg, a_smem, Kd, k, B, ldb, lane, cnt);
+            saxpy_chunk<V, U, SPLIT, true, SHORT, DT>(acc, k, cv, cnt, Dcol, ldd, live, sub);
             k = kn;
             sv = svn;
         }

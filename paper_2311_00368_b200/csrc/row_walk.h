@@ -57,6 +57,7 @@ struct RowChunks {
     B2SP_HD void advance() { at += step; }
     B2SP_HD int count() const { return (int)(end - at < size ? end - at : size); }
     B2SP_HD unsigned next(int i) const { return at + step + i; }   // entry i of the warp's next chunk (behind the row: not < end)
+    B2SP_HD int behind() const { return (int)(end - at) - (int)step; }   // entries of the row from the next chunk on (0 or less: none)
 };
 
 }  // namespace b2sp

@@ -63,8 +63,10 @@ extern "C" int row_chunks(int beg, int end, int warps, int size, unsigned char *
         for (RowChunks r(beg, end, warp, warps, size); r.more(); r.advance()) {
             if (++iterations > (end - beg) / size + 1) return 0;
             for (int i = 0; i < (int)r.count(); ++i) taken[(long long)r.at + i - beg] += 1;
-            for (int lane = 0; lane < 32; ++lane)
-                if (r.next(lane) < r.end && ((long long)r.next(lane) < beg || (long long)r.next(lane) >= end)) return 0;
+            for (int lane = 0; lane < 32; ++lane) {
+                const bool inside = (long long)r.at + warps * size + lane < end;
+                if ((r.next(lane) < r.end) != inside || (lane < r.behind()) != inside) return 0;
+            }
         }
     }
     return 1;
