@@ -188,8 +188,10 @@ b2sp_status pattern_pass(bool prepared, int M, int K, long long nnz, const int *
     const size_t row_bytes = sizeof(unsigned) * (size_t)masks_row_words(Wk);
     // A warp per row wins from about 2000 rows on (2048 x 2048 at 20%: 7.8 against 8.4 us; 1024 x 8192 at 30%: 16.5 against
     // 10.4; 32768 x 8192 at 20%: 62 against 85) unless the rows are long (average 2457 entries on 8192 x 8192: 35.4 against
-    // 31.2 us, 6553 on 4096 x 65536: 71 against 43; 1638 on 32768 x 8192: see above).
-    const bool shared = row_bytes * kMasksRows > kMasksMaxSmem || rows_all < 2000 || nnz / M > 2048;
+    // 31.2 us, 6553 on 4096 x 65536: 71 against 43; 1638 on 32768 x 8192: see above) or wide: with the words of eight rows in
+    // 64 KB of shared memory or less at least 24 warps share an SM (8192 x 65536 at 1%: 41 us, 44 with four warps per row and one load
+    // at a time), beyond that 16 (4096 x 98304 at 1%: 36.9 against 30.9; 2500 x 98304: 29.8 against 18.5).
+    const bool shared = row_bytes * kMasksRows > 64 * 1024 || rows_all < 2000 || nnz / M > 2048;
     auto launch = [&](auto kernel, long long blocks, int threads, size_t smem) {
         const long long cap = 1ll << 24;
         kernel<<<(unsigned)(blocks < cap ? blocks : cap), threads, smem, st>>>(M, K, Wk, nnz, row_ptr, col_idx, win, flags, sig, sig_dev);

@@ -68,6 +68,21 @@ def test_table_entries(b, M, K, shift):
     assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
 
 
+@pytest.mark.parametrize("M,K", [(2001, 65536), (2001, 65537), (2001, 98304), (2001, 98305)])
+def test_table_entries_of_wide_patterns(b, M, K):
+    """Either side of the widths at which eight rows' words no longer fit in a block's share of the shared memory."""
+    rng = np.random.default_rng(K)
+    lens = [int(rng.integers(0, 60)) if i % 50 else 2100 for i in range(M)]
+    rp, ci = make_rows(rng, lens, K)
+    drp, dci = device(rp, ci, 1)
+    ws = torch.zeros(1 << 26, dtype=torch.uint8, device="cuda")
+    b.prepare_pattern(drp, dci, K, ws)
+    mask, pos = table_of(ws, M, K)
+    want_mask, want_pos = expected(rp, ci, K)
+    assert flags_of(ws) == 0
+    assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
+
+
 @pytest.mark.parametrize("M", [44, 2200])
 @pytest.mark.parametrize("row,entry", [(13, 5), (14, 2045), (17, 2048), (20, 2304), (21, 2899), (21, 2050), (9, 255)])
 def test_disorder_is_seen_wherever_it_is(b, M, row, entry):
