@@ -148,15 +148,18 @@ def workspace_bytes(op: int, M: int, K: int, Kd: int, N: int, nnz: int, algo=Non
 _ws_cache = {}
 
 
-# Sizes only; emptied by the debug hooks that change the planner's choice.
+_planner_setting = 0   # counts the calls of the debug hooks that change the planner's choice
+
+
+# Sizes only, by the planner's setting: a size that another thread asked for while a hook took effect is not met again.
 @functools.lru_cache(maxsize=4096)
-def _workspace_need(op, M, K, Kd, N, nnz, algo):
+def _workspace_need(op, M, K, Kd, N, nnz, algo, setting):
     return workspace_bytes(op, M, K, Kd, N, nnz, algo)
 
 
 def _workspace(op, M, K, Kd, N, nnz, device, workspace, algo=0):
     if workspace is None:
-        need = _workspace_need(op, M, K, Kd, N, nnz, algo)
+        need = _workspace_need(op, M, K, Kd, N, nnz, algo, _planner_setting)
         key = (device.index, _raw_stream(device.index))
         workspace = _ws_cache.get(key)
         if workspace is None or workspace.numel() < need:
@@ -192,14 +195,16 @@ def last_launches(op: int) -> int:
 
 def debug_force_k_splits(k_splits: int) -> None:
     """b2sp_debug_force_k_splits: override the dense-tile planner's K split (0 = planner's choice)."""
-    _workspace_need.cache_clear()
+    global _planner_setting
     lib.b2sp_debug_force_k_splits(int(k_splits))
+    _planner_setting += 1
 
 
 def debug_force_partition(partition: int) -> None:
     """b2sp_debug_force_partition: 0 = planner's choice, 1 = tiles x K splits only, 2 = balanced wherever offered."""
-    _workspace_need.cache_clear()
+    global _planner_setting
     lib.b2sp_debug_force_partition(int(partition))
+    _planner_setting += 1
 
 
 def debug_inject_wait_timeout(chunk: int, limit_ns: int = 0) -> None:
