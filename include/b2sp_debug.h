@@ -75,6 +75,15 @@ void b2sp_debug_force_partition(int partition);
  */
 b2sp_status b2sp_debug_inject_wait_timeout(int chunk, unsigned long long limit_ns);
 
+/*
+ * Where b2sp_prepare_pattern leaves things in a workspace, in bytes: the window table of a pattern of M rows (for every row and
+ * every 32-column window {first position, occupancy mask}, two ints; the tables of a batch follow one another), and the int
+ * that is not 0 when the table cannot be used because a row's columns are not strictly increasing or out of range.
+ * For tests that look at the table itself.
+ */
+size_t b2sp_debug_window_table_offset(int M);
+size_t b2sp_debug_unsorted_flag_offset(void);
+
 #ifdef __cplusplus
 }
 #endif

@@ -87,6 +87,10 @@ lib.b2sp_debug_force_k_splits.restype = None
 lib.b2sp_debug_force_k_splits.argtypes = [_i]
 lib.b2sp_debug_force_partition.restype = None
 lib.b2sp_debug_force_partition.argtypes = [_i]
+lib.b2sp_debug_window_table_offset.restype = _sz
+lib.b2sp_debug_window_table_offset.argtypes = [_i]
+lib.b2sp_debug_unsorted_flag_offset.restype = _sz
+lib.b2sp_debug_unsorted_flag_offset.argtypes = []
 lib.b2sp_debug_inject_wait_timeout.restype = _i
 lib.b2sp_debug_inject_wait_timeout.argtypes = [_i, ctypes.c_ulonglong]
 
@@ -205,6 +209,16 @@ def debug_force_partition(partition: int) -> None:
     global _planner_setting
     lib.b2sp_debug_force_partition(int(partition))
     _planner_setting += 1
+
+
+def debug_window_table_offset(M: int) -> int:
+    """b2sp_debug_window_table_offset: where the window table of a pattern of M rows begins in a workspace, in bytes."""
+    return int(lib.b2sp_debug_window_table_offset(M))
+
+
+def debug_unsorted_flag_offset() -> int:
+    """b2sp_debug_unsorted_flag_offset: the int of a workspace that says that its window table cannot be used."""
+    return int(lib.b2sp_debug_unsorted_flag_offset())
 
 
 def debug_inject_wait_timeout(chunk: int, limit_ns: int = 0) -> None:

@@ -512,6 +512,10 @@ extern "C" void b2sp_debug_force_partition(int partition)
     b2sp::g_forced_partition.store(partition == 1 || partition == 2 ? partition : 0, std::memory_order_relaxed);
 }
 
+// Declared in include/b2sp_debug.h.
+extern "C" size_t b2sp_debug_window_table_offset(int M) { return b2sp::pattern_table_offset(M); }
+extern "C" size_t b2sp_debug_unsorted_flag_offset(void) { return b2sp::kWsTileFlagsOffset + sizeof(int) * b2sp::kFlagUnsorted; }
+
 // Debug hook declared in include/b2sp_debug.h.
 extern "C" b2sp_status b2sp_debug_inject_wait_timeout(int chunk, unsigned long long limit_ns)
 {

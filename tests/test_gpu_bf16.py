@@ -106,7 +106,7 @@ def every_family(b, p, ops=("spmm", "sddmm", "fusedmm"), tile=True):
     (512, 2048, 0.10, 128, 256, "uniform"),   # several K splits
     (384, 1024, 0.20, 64, 128, "powerlaw"),   # skewed rows incl. full rows
     (256, 512, 0.20, 32, 32, "band"),
-    (260, 700, 0.20, 48, 63, "uniform"),      # odd width: scalar row kernels, plain stores in the tile flush
+    (260, 700, 0.20, 48, 63, "uniform"),      # odd width: single-element loads in the row kernels, plain stores in the tile flush
     (65, 700, 0.30, 260, 512, "uniform"),     # Kd > 128: row kernels only (A row in shared memory)
 ])
 def test_bf16_shapes_every_family(b, M, K, density, Kd, N, kind):

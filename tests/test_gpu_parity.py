@@ -109,8 +109,8 @@ def test_hand_worked_integer_example_exact(b):
     (33, 260, 0.3, 132, 644, "uniform"),     # N > 512: two column slabs, ragged second slab
     (200, 256, 0.2, 128, 256, "powerlaw"),   # skewed rows incl. saturated rows
     (128, 256, 0.2, 64, 64, "band"),
-    (31, 97, 0.3, 7, 5, "uniform"),          # odd widths: scalar kernels
-    (64, 128, 0.3, 130, 130, "uniform"),     # widths = 2 mod 4: scalar kernels
+    (31, 97, 0.3, 7, 5, "uniform"),          # odd widths: single-element loads
+    (64, 128, 0.3, 130, 130, "uniform"),     # widths = 2 mod 4: loads of pairs
     (1, 64, 0.5, 16, 16, "uniform"),         # single row
 ])
 def test_small_shapes(b, M, K, density, Kd, N, kind):
@@ -183,7 +183,7 @@ def test_leading_dimensions_and_inplace_sddmm(b):
     ref, T = oracle.spmm(p.row_ptr, p.col_idx, p.values, p.D)
     b.spmm(d.row_ptr, d.col_idx, d.values, D, out=out)
     gate(out, ref, T, "spmm ld")
-    # odd leading dimension -> scalar path
+    # odd leading dimension: single-element loads
     D3 = pad(d.D, 3)
     b.spmm(d.row_ptr, d.col_idx, d.values, D3, out=out)
     gate(out, ref, T, "spmm odd ld")

@@ -76,3 +76,30 @@ def test_batched_row_kernels_at_any_alignment(b, dtype, Kd, N):
     for i, p in enumerate(probs):
         hA, hB, hD = (t.float().numpy() for t in host[i])
         gate(out[i], *oracle.fusedmm(p.row_ptr, p.col_idx, p.values, hA, hB, hD), f"problem {i}")
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("Kd,N,pad,shift", [
+    (12289, 5, 0, 0), (12290, 6, 0, 0), (12292, 8, 0, 0), (13001, 33, 0, 0),   # more than 48 KB of shared memory for A_i
+    (40960, 8, 0, 0), (40960, 6, 2, 2), (40959, 5, 0, 1),                       # the longest that is staged there
+    (40961, 5, 0, 0), (40964, 132, 0, 0),                                       # a lane per dot product
+])
+def test_long_dot_products(b, dtype, Kd, N, pad, shift):
+    nb, M, K = 2, 9, 40
+    probs = [W.small_random(7200 + Kd % 97 + i, M, K, 0.3, Kd, N) for i in range(nb)]
+    most = max(p.nnz for p in probs)
+    fill = lambda x: np.pad(x, (0, most - x.size))
+    rp = torch.from_numpy(np.stack([p.row_ptr for p in probs])).cuda()
+    ci, v = (torch.from_numpy(np.stack([fill(x) for x in xs])).cuda() for xs in ([p.col_idx for p in probs], [p.values for p in probs]))
+    host = [[torch.from_numpy(x).to(dtype).float().numpy() for x in (p.A, p.B, p.D)] for p in probs]
+    refs = [oracle.fusedmm(p.row_ptr, p.col_idx, p.values, *h) for p, h in zip(probs, host)]
+    for i, (p, h) in enumerate(zip(probs, host)):
+        dA, dB, dD = (strided(x, dtype, pad, shift) for x in h)
+        sd = oracle.sddmm(p.row_ptr, p.col_idx, p.values, h[0], h[1])
+        for algo in (ROW, ROW_NAT):
+            gate(b.fusedmm(rp[i], ci[i, :p.nnz], v[i, :p.nnz], dA, dB, dD, algo=algo, dtype=dtype), *refs[i], f"fusedmm algo={algo}")
+            gate(b.sddmm(rp[i], ci[i, :p.nnz], v[i, :p.nnz], dA, dB, algo=algo, dtype=dtype), *sd, f"sddmm algo={algo}")
+    A, B, D = (torch.stack([torch.from_numpy(h[j]).to(dtype) for h in host]).cuda() for j in range(3))
+    out = b.fusedmm_batched(rp, ci, v, A, B, D, algo=ROW, dtype=dtype)
+    for i in range(nb):
+        gate(out[i], *refs[i], f"problem {i}")

@@ -33,16 +33,15 @@ def expected(rp, ci, K):
     return mask, rp[:-1, None] + np.cumsum(count, 1) - count
 
 
-def table_of(ws, M, K, batch=1):
-    off = (512 + 4 * M + 255) // 256 * 256
-    off = (off + 1023) // 1024 * 1024
-    Wk = (K + 31) // 32
+def table_of(b, ws, M, K, batch=1):
+    off, Wk = b.debug_window_table_offset(M), (K + 31) // 32
     t = ws[off:off + 8 * batch * M * Wk].view(torch.int32).cpu().numpy().reshape(batch, M, Wk, 2)
     return t[..., 1].view(np.uint32), t[..., 0]
 
 
-def flags_of(ws):
-    return int(ws[320:324].view(torch.int32).item())
+def flag_of(b, ws):
+    off = b.debug_unsorted_flag_offset()
+    return int(ws[off:off + 4].view(torch.int32).item())
 
 
 def device(rp, ci, shift):
@@ -62,9 +61,23 @@ def test_table_entries(b, M, K, shift):
     drp, dci = device(rp, ci, shift)
     ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
     b.prepare_pattern(drp, dci, K, ws)
-    mask, pos = table_of(ws, M, K)
+    mask, pos = table_of(b, ws, M, K)
     want_mask, want_pos = expected(rp, ci, K)
-    assert flags_of(ws) == 0
+    assert flag_of(b, ws) == 0
+    assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
+
+
+@pytest.mark.parametrize("M,K,length", [(2100, 2999, 2500), (2100, 2999, 2047), (2100, 2999, 2049), (2000, 4096, 2100), (1999, 4096, 2100)])
+def test_table_entries_of_many_long_rows(b, M, K, length):
+    """Either side of the average length and the number of rows at which four warps share a row."""
+    rng = np.random.default_rng(M + length)
+    rp, ci = make_rows(rng, [length + (i % 3) - 1 for i in range(M)], K)
+    drp, dci = device(rp, ci, 3)
+    ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
+    b.prepare_pattern(drp, dci, K, ws)
+    mask, pos = table_of(b, ws, M, K)
+    want_mask, want_pos = expected(rp, ci, K)
+    assert flag_of(b, ws) == 0
     assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
 
 
@@ -77,20 +90,25 @@ def test_table_entries_of_wide_patterns(b, M, K):
     drp, dci = device(rp, ci, 1)
     ws = torch.zeros(1 << 26, dtype=torch.uint8, device="cuda")
     b.prepare_pattern(drp, dci, K, ws)
-    mask, pos = table_of(ws, M, K)
+    mask, pos = table_of(b, ws, M, K)
     want_mask, want_pos = expected(rp, ci, K)
-    assert flags_of(ws) == 0
+    assert flag_of(b, ws) == 0
     assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
 
 
 @pytest.mark.parametrize("M", [44, 2200])
-@pytest.mark.parametrize("row,entry", [(13, 5), (14, 2045), (17, 2048), (20, 2304), (21, 2899), (21, 2050), (9, 255)])
+@pytest.mark.parametrize("row,entry", [(13, 5), (14, 2045), (17, 2048), (20, 2304), (21, 2899), (21, 2050), (9, 255),
+                                       (17, "seam"), (20, "seam"), (21, "seam"), (21, "after the seam"), (20, "before the seam")])
 def test_disorder_is_seen_wherever_it_is(b, M, row, entry):
-    """Two entries of a row swapped, a repeated entry, a column out of range: each raises the flag."""
-    rng = np.random.default_rng(row + entry)
+    """Two entries of a row swapped, a repeated entry, a column out of range: each raises the flag.  The seam is the first entry of
+    a row that its own warp leaves to the block: 2048 entries after the 16-byte boundary at or before the row."""
+    rng = np.random.default_rng([row, len(str(entry))])
     K = 2999
     lens = EDGE_LENS * (M // len(EDGE_LENS)) if M < 100 else EDGE_LENS + [100] * (M - len(EDGE_LENS))
     rp, ci = make_rows(rng, lens, K)
+    if isinstance(entry, str):
+        begin = int(rp[row]) + 1   # (the arrays begin one element behind a boundary)
+        entry = begin // 4 * 4 + 2048 - begin + {"seam": 0, "after the seam": 1, "before the seam": -1}[entry]
     p = int(rp[row]) + min(entry, lens[row] - 1)
     ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
     for what in ("swap", "repeat", "below", "above"):
@@ -103,25 +121,30 @@ def test_disorder_is_seen_wherever_it_is(b, M, row, entry):
             bad[p] = -1 if what == "below" else K
         drp, dci = device(rp, bad, 1)
         b.prepare_pattern(drp, dci, K, ws)
-        assert flags_of(ws) == 1, what
+        assert flag_of(b, ws) == 1, what
     drp, dci = device(rp, ci, 1)
     b.prepare_pattern(drp, dci, K, ws)
-    assert flags_of(ws) == 0
+    assert flag_of(b, ws) == 0
 
 
-@pytest.mark.parametrize("batch,M,K", [(3, 30, 700), (7, 333, 257)])
-def test_batched_tables(b, batch, M, K):
+@pytest.mark.parametrize("batch,M,K,long", [(3, 30, 700, 0), (7, 333, 257, 0), (5, 500, 4096, 3000), (3, 700, 2600, 2600)])
+def test_batched_tables(b, batch, M, K, long):
+    """Also with 2000 rows or more in all and some of them longer than a warp's own share, in every problem."""
     rng = np.random.default_rng(batch)
-    probs = [make_rows(rng, [int(rng.integers(0, min(K, 256))) for _ in range(M)], K) for _ in range(batch)]
+    probs = [make_rows(rng, [long - i % 7 if long and i % 60 == 7 else int(rng.integers(0, min(K, 256))) for i in range(M)], K)
+             for _ in range(batch)]
     stride = max(ci.size for _, ci in probs) | 1   # odd: most problems begin off a 16-byte boundary
-    ci = np.full((batch, stride), -1, np.int32)
+    # (the last problem's array ends with its last entry, and what lies behind it would break the order if it were read as its own)
+    ci = np.full((batch - 1) * stride + probs[-1][1].size, -1, np.int32)
     for i, (_, c) in enumerate(probs):
-        ci[i, :c.size] = c
+        ci[i * stride:i * stride + c.size] = c
     rp = np.stack([r for r, _ in probs])
     ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
-    b.prepare_pattern_batched(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), K, ws)
-    mask, pos = table_of(ws, M, K, batch)
-    assert flags_of(ws) == 0
+    flat = torch.full((ci.size + 64,), -1, dtype=torch.int32, device="cuda")
+    flat[:ci.size] = torch.from_numpy(ci)
+    b.prepare_pattern_batched(torch.from_numpy(rp).cuda(), flat.as_strided((batch, 1), (stride, 1)), K, ws)
+    mask, pos = table_of(b, ws, M, K, batch)
+    assert flag_of(b, ws) == 0
     for i, (r, c) in enumerate(probs):
         want_mask, want_pos = expected(r, c, K)
         assert np.array_equal(mask[i], want_mask) and np.array_equal(pos[i], want_pos)
