@@ -18,6 +18,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "row_walk.h"
 
 namespace b2sp {
@@ -362,40 +364,68 @@ __device__ __forceinline__ float sddmm_chunk(const VecF<V> (&areg)[KU > 0 ? KU :
 {
     const int g = lane >> 3, t = lane & 7;
     float mine = 0.f;
-    auto round = [&](int r) {
-        const int kq = __shfl_sync(kFull, k, 4 * r + g);
-        const DT *b = B + (int64_t)kq * ldb + t * V;
-        float part = 0.f;
-        if (KU > 0) {
-#pragma unroll
-            for (int u = 0; u < KU; ++u)
-                if ((t + 8 * u) * V < Kd) part = dot_v<V>(areg[u], ldgv<V>(b + u * 8 * V), part);
-        } else {
-            for (int e = t * V; e < Kd; e += 8 * V)
-                part = dot_v<V>(*reinterpret_cast<const VecF<V> *>(a_smem + e), ldgv<V>(b + e - t * V), part);
-        }
+    auto keep = [&](int r, float part) {
         part += __shfl_xor_sync(kFull, part, 1);
         part += __shfl_xor_sync(kFull, part, 2);
         part += __shfl_xor_sync(kFull, part, 4);
         if (r == t) mine = part;
     };
-    if constexpr (!SHORT) {   // (rounds behind the end of the row read row 0 of B)
-#pragma unroll 4
-        for (int r = 0; r < 8; ++r) round(r);
-    } else if constexpr (!FUSED && KU == 8 && sizeof(DT) == 4) {
-        // four rounds at a time and no second loop: with it 128 < Kd <= 256 took longer than with eight rounds for every chunk,
-        // this way less (4096 x 1024 at 20%, Kd = 256: 73.0, 68.2 and 59.9 us; rows of 40 entries: 19.1, 34.9 and 20.9)
-#pragma unroll 1
-        for (int r0 = 0; 4 * r0 < cnt; r0 += 4) {
+    if constexpr (KU == 0) {
+        // Long dot products: R rounds go through the elements together, so that their loads are in flight at the same time and
+        // A_i is read from shared memory once for all of them.  Round after round, with whatever loads the compiler then kept in
+        // flight: 300 x 300 at 20%, Kd = 8000 sddmm 272 us, now 125; 4000 x 500 at 30%, Kd = 1024 230 and 149; with the elements
+        // unrolled by two instead of four 144 and 157.
+        auto rounds = [&](auto count, int r) {
+            constexpr int R = decltype(count)::value;
+            const DT *b[R];
+            float part[R];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) round(r0 + r);
-        }
-    } else if (cnt == 32) {
+            for (int i = 0; i < R; ++i) {
+                b[i] = B + (int64_t)__shfl_sync(kFull, k, 4 * (r + i) + g) * ldb;
+                part[i] = 0.f;
+            }
 #pragma unroll 4
-        for (int r = 0; r < 8; ++r) round(r);
-    } else {   // (one loop for both, its length known only at run time, cost full chunks a quarter of their speed)
+            for (int e = t * V; e < Kd; e += 8 * V) {
+                const VecF<V> a = *reinterpret_cast<const VecF<V> *>(a_smem + e);
+#pragma unroll
+                for (int i = 0; i < R; ++i) part[i] = dot_v<V>(a, ldgv<V>(b[i] + e), part[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < R; ++i) keep(r + i, part[i]);
+        };
+        const int all = (cnt + 3) >> 2;
+        int r = 0;
+        for (; r + 4 <= all; r += 4) rounds(std::integral_constant<int, 4>(), r);
+        for (; r + 2 <= all; r += 2) rounds(std::integral_constant<int, 2>(), r);
+        if (r < all) rounds(std::integral_constant<int, 1>(), r);
+    } else {
+        auto round = [&](int r) {
+            const int kq = __shfl_sync(kFull, k, 4 * r + g);
+            const DT *b = B + (int64_t)kq * ldb + t * V;
+            float part = 0.f;
+#pragma unroll
+            for (int u = 0; u < KU; ++u)
+                if ((t + 8 * u) * V < Kd) part = dot_v<V>(areg[u], ldgv<V>(b + u * 8 * V), part);
+            keep(r, part);
+        };
+        if constexpr (!SHORT) {   // (rounds behind the end of the row read row 0 of B)
+#pragma unroll 4
+            for (int r = 0; r < 8; ++r) round(r);
+        } else if constexpr (!FUSED && KU == 8 && sizeof(DT) == 4) {
+            // four rounds at a time and no second loop: with it 128 < Kd <= 256 took longer than with eight rounds for every chunk,
+            // this way less (4096 x 1024 at 20%, Kd = 256: 73.0, 68.2 and 59.9 us; rows of 40 entries: 19.1, 34.9 and 20.9)
+#pragma unroll 1
+            for (int r0 = 0; 4 * r0 < cnt; r0 += 4) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) round(r0 + r);
+            }
+        } else if (cnt == 32) {
+#pragma unroll 4
+            for (int r = 0; r < 8; ++r) round(r);
+        } else {   // (one loop for both, its length known only at run time, cost full chunks a quarter of their speed)
 #pragma unroll 2
-        for (int r = 0; r < (cnt + 3) >> 2; ++r) round(r);
+            for (int r = 0; r < (cnt + 3) >> 2; ++r) round(r);
+        }
     }
     return mine;  // lane 8g+t: dot product of entry 4t+g
 }

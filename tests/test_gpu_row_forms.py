@@ -55,7 +55,7 @@ def test_spmm(b, line, M, N, extra, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("extra", [0, 1])
-@pytest.mark.parametrize("Kd", [4, 32, 64, 132, 256])
+@pytest.mark.parametrize("Kd", [4, 32, 64, 132, 256, 257, 258, 260, 516])
 def test_sddmm(b, Kd, extra, dtype):
     rng = np.random.default_rng(Kd + extra)
     rp, ci, v = pattern(rng, 60, 300, 128, extra)
@@ -68,7 +68,7 @@ def test_sddmm(b, Kd, extra, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("extra", [0, 1])
-@pytest.mark.parametrize("Kd,N", [(64, 32), (60, 64), (64, 100), (64, 256), (128, 128), (128, 256), (128, 512), (100, 516), (256, 256), (160, 132)])
+@pytest.mark.parametrize("Kd,N", [(64, 32), (60, 64), (64, 100), (64, 256), (128, 128), (128, 256), (128, 512), (100, 516), (256, 256), (160, 132), (260, 64), (301, 33)])
 def test_fusedmm(b, Kd, N, extra, dtype):
     rng = np.random.default_rng(Kd + N + extra)
     line = 72 if N * dtype.itemsize <= 128 else 144
