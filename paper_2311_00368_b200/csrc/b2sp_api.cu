@@ -478,13 +478,13 @@ static b2sp_status sddmm_rows(int M, int Kd, long long nnz, const int *row_ptr, 
                               float *out_values, const int *order, int *gate, int *clear, cudaStream_t st)
 {
     dim3 grid((unsigned)M);
-    if (Kd > kMaxStagedKd) {
+    const int V = std::min(vec_width(A, Kd, lda), vec_width(B, Kd, ldb));
+    if (Kd > max_staged_kd(V)) {
         grid.x = gated_blocks(grid.x, gate);
         launch_row(sddmm_row_scalar_kernel<DT>, grid, 0, st, gate != nullptr || order != nullptr, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb,
                    out_values, order, gate, M, clear);
         return check_launch();
     }
-    const int V = std::min(vec_width(A, Kd, lda), vec_width(B, Kd, ldb));
     const b2sp_status rc =
         V == 4 ? dispatch_sddmm_ku<4, DT>(sddmm_short(nnz, M), grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
         : V == 2 ? dispatch_sddmm_ku<2, DT>(sddmm_short(nnz, M), grid, st, Kd, row_ptr, col_idx, s_values, A, lda, B, ldb, out_values, order, gate, clear)
@@ -557,13 +557,13 @@ static b2sp_status fused_rows(int M, int Kd, int N, long long nnz, const int *ro
                               int nbatch = 1, const RowBatch &rb = RowBatch{0, 0, 0, 0, 0, 0})
 {
     b2sp_status rc = B2SP_OK;
-    if (Kd > kMaxStagedKd) {
+    const int V = std::min({vec_width(A, Kd, lda, rb.A), vec_width(B, Kd, ldb, rb.B), vec_width(D, N, ldd, rb.D), vec_width(O, N, ldo, rb.O)});
+    if (Kd > max_staged_kd(V)) {
         dim3 grid(gated_blocks((unsigned)M, gate, (unsigned)nbatch), (unsigned)((N + 127) / 128), (unsigned)nbatch);
         launch_row(fusedmm_row_scalar_kernel<DT>, grid, 0, st, gate != nullptr || order != nullptr, Kd, N, row_ptr, col_idx, s_values, A, lda, B, ldb,
                    D, ldd, O, ldo, order, gate, M, clear, rb);
         return check_launch();
     }
-    const int V = std::min({vec_width(A, Kd, lda, rb.A), vec_width(B, Kd, ldb, rb.B), vec_width(D, N, ldd, rb.D), vec_width(O, N, ldo, rb.O)});
     const Geom g = pick_geom(N, V);
     dim3 grid((unsigned)M, (unsigned)((N + g.slab - 1) / g.slab), (unsigned)nbatch);
     const bool is_short = fused_short<DT>(nnz, M, N);

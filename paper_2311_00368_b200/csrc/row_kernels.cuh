@@ -28,7 +28,11 @@ constexpr int kRowWarps = 4;
 constexpr int kRowThreads = kRowWarps * 32;
 constexpr int kBuckets = 32;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kMaxStagedKd = 40960;   // longest A_i that is staged in shared memory
+// Longest A_i that is staged in shared memory, by the elements that a load takes.  Fewer than four mean two to four times as many
+// loads, and then the few CTAs that fit on an SM beside a long A_i lose to a lane per entry (us, staged and a lane per entry, 2000 x
+// 2000 at 2%: Kd = 16001 sddmm 2850 and 3520, 20001 5000 and 4500, 20002 2580 and 4320, 30002 7940 and 6510; N = 33 fusedmm 16001
+// 2720 and 3630, 30001 14700 and 6680; N = 34 20002 2760 and 4160, 30002 8340 and 6260).
+__host__ __device__ constexpr int max_staged_kd(int V) { return V == 4 ? 40960 : V == 2 ? 24576 : 16384; }
 
 // ------------------------------------------------------------------------------------------
 // Row binning (work assignment): counting sort of the rows by length bucket
@@ -478,7 +482,7 @@ sddmm_row_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict_
     }
 }
 
-// Kd too long for A_i in shared memory (kMaxStagedKd): one lane per entry, serial dot product.
+// Kd too long for A_i in shared memory (max_staged_kd): one lane per entry, serial dot product.
 template <typename DT>
 __global__ void __launch_bounds__(kRowThreads)
 sddmm_row_scalar_kernel(int Kd, const int *__restrict__ row_ptr, const int *__restrict__ col_idx,

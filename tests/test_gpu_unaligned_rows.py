@@ -81,8 +81,9 @@ def test_batched_row_kernels_at_any_alignment(b, dtype, Kd, N):
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("Kd,N,pad,shift", [
     (12289, 5, 0, 0), (12290, 6, 0, 0), (12292, 8, 0, 0), (13001, 33, 0, 0),   # more than 48 KB of shared memory for A_i
-    (40960, 8, 0, 0), (40960, 6, 2, 2), (40959, 5, 0, 1),                       # the longest that is staged there
-    (40961, 5, 0, 0), (40964, 132, 0, 0),                                       # a lane per dot product
+    (16384, 5, 1, 0), (16383, 6, 0, 1), (24576, 6, 0, 2), (40960, 8, 0, 0),     # the longest that are staged there
+    (16385, 5, 0, 0), (16388, 6, 1, 0), (24578, 130, 0, 0), (24580, 6, 2, 2),   # a lane per dot product
+    (40961, 5, 0, 0), (40964, 132, 0, 0),
 ])
 def test_long_dot_products(b, dtype, Kd, N, pad, shift):
     nb, M, K = 2, 9, 40
