@@ -168,9 +168,10 @@ b2sp_status b2sp_fusedmm(int M, int K, int Kd, int N, long long nnz,
  * Eq. 1-3 evaluated exactly on the bfloat16 values: every product of two bfloat16 numbers is exact in
  * fp32, only the order of the fp32 sums differs.  The row kernels gather half the bytes per dense row;
  * the dense-tile kernels need no lo halves for operands that are exact in tf32, i.e. one tensor-core
- * product per GEMM1 term instead of three and two per GEMM2 term.  The four-element loads of the vector
- * kernels want 8-byte aligned operands and leading dimensions that are multiples of 4 (16 bytes and
- * multiples of 8 for A on the dense-tile kernels); other shapes take the scalar paths.
+ * product per GEMM1 term instead of three and two per GEMM2 term.  The row kernels load
+ * four elements at a time where every operand's address, width and leading dimension is a multiple of
+ * four elements, two where all are even, single ones otherwise (A on the dense-tile kernels: eight-element
+ * loads where it is 16-byte aligned with a leading dimension that is a multiple of 8).
  */
 b2sp_status b2sp_spmm_bf16(int M, int K, int N, long long nnz,
                            const int *row_ptr, const int *col_idx, const float *values,

@@ -127,7 +127,8 @@ void launch_spmm(dim3 grid, cudaStream_t st, int N, const int *row_ptr, const in
 
 // Column geometry for a width N: U groups of V columns per lane, SPLIT sub-warps.
 // (V < 4, rows that are not aligned groups of four: loads of two or one elements are two to four times as many, but even the
-// single ones beat a lane per dot product: 1501 x 2903 at 12%, fusedmm Kd = 51, N = 71 68 -> 42 us, Kd = 50, N = 70 71 -> 37 us.)
+// single ones beat a lane per dot product: 1501 x 2903 at 12%, fusedmm Kd = 51, N = 71 68 -> 42 us, Kd = 50, N = 70 71 -> 37 us,
+// on the device alone.  SPMM with 65 to 128 columns and 100 to 350 entries a row is 4% to 6% slower: x 70 23.6 -> 24.8 us.)
 struct Geom { int U, SPLIT, slab; };
 inline Geom pick_geom(int N, int V)
 {
@@ -299,10 +300,11 @@ extern "C" const char *b2sp_status_string(b2sp_status s)
 // writing the sampled values once: measured at N = 512 on the 8192^2 / 30% workload, 717 us fused
 // against 134 + 430 us for SDDMM into a scratch C and SPMM on C.  So wide outputs take the two
 // phases inside one call (same window table, same fallback), and C lives in the workspace.
-// With two tiles (128 < N <= 256) the second GEMM1 costs more than C's round trip when GEMM1 is long and the
-// problem large: measured at N = 256, Kd = 128, two phases against fused: 8192^2 315 against 342 us (10% density
-// 298 against 337), 4096 x 8192 175 against 188, 16384 x 2048 187 against 191, 4096^2 115 against 114; but
-// 8192 x 4096 at Kd = 64 172 against 159 and 2048^2 52 against 40.
+// With two tiles (128 < N <= 256) the second GEMM1 costs about what C's round trip does when GEMM1 is long and the
+// problem large: measured at N = 256, Kd = 128, two phases against fused: 8192^2 286 against 288 us (10% density
+// 270 against 279), 4096 x 8192 158 against 153, 16384 x 2048 171 against 152, 4096^2 92 against 85;
+// 8192 x 4096 at Kd = 64 156 against 122 and 2048^2 46 against 33.  (The line was drawn on an earlier fused kernel, 342 us at
+// 8192^2; the largest problems are what is left of its reason.)
 static bool fusedmm_two_phase(int M, int K, int Kd, int N)
 {
     return N > 256 || (N > 128 && Kd > 64 && (double)M * (double)K >= 3.0e7);

@@ -131,8 +131,8 @@ int pick_balanced(long long units, int nt, int blocks, int ks, int mode, int *sl
         // A CTA that goes on into the next row tile reloads its A tile (FusedMM, SDDMM: about a block and a half of
         // time).  Measured: the time falls by about 0.6 of what the lengths promise (more CTAs at work slow each other
         // down), and slabs where the plain partition writes straight into O (one K split) cost a few percent.  At 7/8 of
-        // the length: 8192^2 x 128 SPMM -7%, FusedMM -3%, SDDMM -3%; x 256 (one K split) SPMM -4%, FusedMM -1%; 4096^2
-        // SDDMM (8 -> 7 blocks per CTA) +3%.  At 2/3 (24576 x 8192, 192 row tiles): -27% / -26% / -27%.
+        // the length: 8192^2 x 128 SPMM -7%, FusedMM -7%, SDDMM -3%; x 256 (one K split) SPMM -5%; 4096^2
+        // SDDMM (8 -> 7 blocks per CTA) +9%.  At 2/3 (24576 x 8192, 192 row tiles): -28% / -33% / -30%.
         const long long plain2 = 2 * ((units * nt * ks + kSMs - 1) / kSMs * ((blocks + ks - 1) / ks));
         const long long mine2 = 2 * gmax * gran + (mode == kModeSpmm ? 0 : 3);
         // (SPMM on one column tile: slabs where there were none cost more than 1/8 of the length buys -- 16384 x 4096 x 128,
@@ -209,13 +209,15 @@ b2sp_status pattern_pass(bool prepared, int M, int K, long long nnz, const int *
 
 bool tile_profitable(int op, int M, int K, int width, long long nnz)
 {
-    // Measured on B200: the dense-tile family costs a fixed ~35 us (pattern pre-pass, operand splits,
-    // tile prologue) plus ~1.3 us per million cells of S whatever the density, the row family ~22 us
-    // plus ~31 us per million stored entries (width 128).  The cross-over density is therefore about
-    // 4.5% on large matrices and rises as the matrix shrinks (16% at 2048^2, never at 1024^2).
+    // Measured on B200 at width 128: an SPMM of the dense-tile family costs a fixed ~22 us (pattern pre-pass, operand
+    // splits, tile prologue) plus ~1.3 us per million cells of S, nearly whatever the density (1024^2 23 us, 4096^2 43, 8192^2
+    // 106), the row family ~8 us (~25 with the binning pass, above 4096 rows) plus ~26 us per million stored entries.  The
+    // cross-over is between 3.5% and 5% at 8192^2 (SPMM 5%: row 113, tile 106 us), 5% and 8% at 4096^2, 12% and 20% at 2048^2,
+    // above 20% at 1024^2; the fit below, made on earlier kernels, lies in these intervals.
     // Operands narrower than 64 use half of a 64-wide tile at best while the row kernels lose nothing
-    // (sub-warps share a row): measured at width 32 on 1k^2 ... 32k x 8k, the cross-over is about 3.5x
-    // higher for SPMM, 2x for SDDMM, 2.5x for FusedMM.  With 74 or more row tiles (no K split) the last
+    // (sub-warps share a row): at width 32 the cross-over is about 3.5x higher for SPMM, 2x for SDDMM, 2.5x for
+    // FusedMM (8192^2: FusedMM row 87 and tile 112 us at 5%, 123 and 114 at 8%).  Widths of 33 to 63 are charged the same, which
+    // is too much (FusedMM, width 48: 8192^2 at 5% row 128, tile 114; 2048^2 at 20% 36 and 29).  With 74 or more row tiles (no K split) the last
     // wave of CTAs is partly empty (96 tiles: 65% of the SMs; 192 tiles: two waves, 65%), which the tile
     // family pays in full unless the balanced partition applies: the cross-over rises by the waves' efficiency
     // against the usual 86%.

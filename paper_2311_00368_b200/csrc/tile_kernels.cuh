@@ -101,9 +101,9 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
 // starting at 0; col_idx arrays `sig.nz_stride` elements apart) gives one table per pattern, stacked:
 // T[(b*M + r)*Wk + w], positions relative to the pattern's own col_idx array.
 //
-// SHARED = false: a block of eight warps has eight rows, a warp to each, so that no row waits for a block-wide barrier
-// between its steps.  A warp reads the first kMasksOwn entries of its row by itself; what is left of longer rows is dealt to
-// all eight warps, so that a long row is not one warp's chain of iterations.  SHARED = true: the four warps of a block
+// SHARED = false: a block of eight warps has eight rows, a warp to each, which meet once, between the sweeps, to hear whether
+// one of the rows is long: a warp reads the first kMasksOwn entries of its row by itself, and what is left of longer rows is
+// dealt to all eight warps, so that a long row is not one warp's chain of iterations.  SHARED = true: the four warps of a block
 // share one row throughout, for few rows (which would leave the GPU idle otherwise), for long ones and for rows whose words
 // fill the shared memory.
 // What bounds it: instruction issue (82% of the slots at 32768 rows of 820 entries, 2.7 TB/s; about 30 instructions per
