@@ -163,9 +163,13 @@ inline int pick_ku(int Kd, int V)
 // that is missing here is served better, or as well, by the form for short rows over the whole range.
 template <int V, int U, int SPLIT> constexpr bool spmm_has_long() { return V == 4 && (SPLIT == 2 || U >= 2); }
 template <int V, int KU, typename DT> constexpr bool sddmm_has_long() { return V == 4 && (KU == 2 || (KU == 8 && sizeof(DT) == 2)); }
-template <int V, int KU, int U, int SPLIT, typename DT> constexpr bool fused_has_long()
+// (The kernels for batches are others, and so are their registers: four problems of 3877 x 3877 at 267 entries a row, fp32, short and
+// long, Kd = N = 64 151 / 168 us, Kd = 128, N = 512 650 / 736, Kd = N = 256 500 / 706.)
+template <int V, int KU, int U, int SPLIT, bool BATCHED, typename DT> constexpr bool fused_has_long()
 {
-    return V == 4 && (KU == 2 ? U <= 2 : KU == 4 ? SPLIT == 1 : KU == 8 && sizeof(DT) == 4 && U == 2);
+    constexpr bool F32 = sizeof(DT) == 4;
+    return V == 4 && (KU == 2 ? U <= 2 && !(BATCHED && F32 && SPLIT == 2)
+                      : KU == 4 ? SPLIT == 1 && !(BATCHED && F32 && U == 4) : KU == 8 && U == 2 && F32 && !BATCHED);
 }
 inline bool short_rows(long long nnz, int M, int entries) { return nnz <= (long long)entries * M; }
 // x 64: 130 entries 15.0 / 15.3, 300 27.3 / 26.0; power law 8192 x 8192 at 10% 156 / 134.  x 256: 130 entries 31.9 / 33.3, 205
@@ -223,12 +227,13 @@ b2sp_status launch_fused(dim3 grid, cudaStream_t st, int Kd, int N, const int *r
 }
 
 template <int V, int KU, int U, int SPLIT, typename DT, class... Args>
-b2sp_status launch_fused_form(bool is_short, Args... args)
+b2sp_status launch_fused_form(bool is_short, dim3 grid, Args... args)
 {
-    if constexpr (fused_has_long<V, KU, U, SPLIT, DT>()) {
-        if (!is_short) return launch_fused<V, KU, U, SPLIT, false, DT>(args...);
+    constexpr bool one = fused_has_long<V, KU, U, SPLIT, false, DT>(), many = fused_has_long<V, KU, U, SPLIT, true, DT>();
+    if constexpr (one || many) {
+        if (!is_short && (grid.z > 1 ? many : one)) return launch_fused<V, KU, U, SPLIT, false, DT>(grid, args...);
     }
-    return launch_fused<V, KU, U, SPLIT, true, DT>(args...);
+    return launch_fused<V, KU, U, SPLIT, true, DT>(grid, args...);
 }
 
 template <int V, int KU, typename DT, class... Args>
