@@ -299,14 +299,14 @@ TwoPhasePlan plan_two_phase(int M, int K, int Kd, int N, long long nnz, size_t b
 
 namespace {
 
-template <int KDP, int MODE, int PART, bool EXACT>
+template <int KDP, int MODE, int PART, bool EXACT, bool ONES>
 b2sp_status launch_fused_tile(const CUtensorMap &bh, const CUtensorMap &bl, const CUtensorMap &dh,
                               const CUtensorMap &dl, const CUtensorMap &out, const FusedTileArgs &a, int items,
                               cudaStream_t st)
 {
-    using Cfg = FusedCfg<KDP, MODE, EXACT>;
-    auto kern = fused_tile_kernel<KDP, MODE, PART, EXACT>;
-    if (!allow_dynamic_smem<KDP * 32 + MODE * 8 + PART * 2 + (EXACT ? 1 : 0)>(reinterpret_cast<const void *>(kern), Cfg::SMEM_BYTES)) return B2SP_ERR_CUDA;
+    using Cfg = FusedCfg<KDP, MODE, EXACT, ONES>;
+    auto kern = fused_tile_kernel<KDP, MODE, PART, EXACT, ONES>;
+    if (!allow_dynamic_smem<KDP * 64 + MODE * 16 + PART * 4 + (EXACT ? 2 : 0) + (ONES ? 1 : 0)>(reinterpret_cast<const void *>(kern), Cfg::SMEM_BYTES)) return B2SP_ERR_CUDA;
     // a programmatic dependent of the operand-split kernel: its CTAs are placed while that kernel still runs
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)items);
@@ -322,36 +322,44 @@ b2sp_status launch_fused_tile(const CUtensorMap &bh, const CUtensorMap &bl, cons
     return cudaGetLastError() == cudaSuccess ? B2SP_OK : B2SP_ERR_CUDA;
 }
 
-// Picks the instantiation: PART from the plan, EXACT from the operand type, KDP from the padded Kd (SPMM has no A / B:
-// only its KDP = 32 instantiation exists).
-template <int MODE, int PART, bool EXACT>
-b2sp_status launch_fused_part(int kdp, const CUtensorMap &bh, const CUtensorMap &bl, const CUtensorMap &dh, const CUtensorMap &dl,
-                              const CUtensorMap &out, const FusedTileArgs &a, int items, cudaStream_t st)
+// Picks the instantiation: PART from the plan, EXACT from the operand type, ONES (FusedMM without stored values) from the
+// call, KDP from the padded Kd (SPMM has no A / B: only its KDP = 32 instantiation exists).
+template <int MODE, int PART, bool EXACT, bool ONES>
+b2sp_status launch_fused_kdp(int kdp, const CUtensorMap &bh, const CUtensorMap &bl, const CUtensorMap &dh, const CUtensorMap &dl,
+                             const CUtensorMap &out, const FusedTileArgs &a, int items, cudaStream_t st)
 {
     if constexpr (MODE == kModeSpmm) {
-        return launch_fused_tile<32, MODE, PART, EXACT>(bh, bl, dh, dl, out, a, items, st);
+        return launch_fused_tile<32, MODE, PART, EXACT, ONES>(bh, bl, dh, dl, out, a, items, st);
     } else {
-        if (kdp == 32) return launch_fused_tile<32, MODE, PART, EXACT>(bh, bl, dh, dl, out, a, items, st);
-        if (kdp == 64) return launch_fused_tile<64, MODE, PART, EXACT>(bh, bl, dh, dl, out, a, items, st);
-        return launch_fused_tile<128, MODE, PART, EXACT>(bh, bl, dh, dl, out, a, items, st);
+        if (kdp == 32) return launch_fused_tile<32, MODE, PART, EXACT, ONES>(bh, bl, dh, dl, out, a, items, st);
+        if (kdp == 64) return launch_fused_tile<64, MODE, PART, EXACT, ONES>(bh, bl, dh, dl, out, a, items, st);
+        return launch_fused_tile<128, MODE, PART, EXACT, ONES>(bh, bl, dh, dl, out, a, items, st);
     }
 }
 
-template <int MODE>
-b2sp_status launch_fused_kdp(int kdp, bool exact, const CUtensorMap &bh, const CUtensorMap &bl, const CUtensorMap &dh,
-                             const CUtensorMap &dl, const CUtensorMap &out, const FusedTileArgs &a, int items,
-                             cudaStream_t st)
+template <int MODE, int PART, bool EXACT, class... Args>
+b2sp_status launch_fused_ones(bool ones, const Args &...args)
 {
-    if (a.bal_ctas > 0)
-        return exact ? launch_fused_part<MODE, kPartBalanced, true>(kdp, bh, bl, dh, dl, out, a, items, st)
-                     : launch_fused_part<MODE, kPartBalanced, false>(kdp, bh, bl, dh, dl, out, a, items, st);
-    if constexpr (MODE == kModeFused) {   // (only FusedMM is offered on batches)
-        if (a.batch > 1)
-            return exact ? launch_fused_part<MODE, kPartBatched, true>(kdp, bh, bl, dh, dl, out, a, items, st)
-                         : launch_fused_part<MODE, kPartBatched, false>(kdp, bh, bl, dh, dl, out, a, items, st);
-    }
-    return exact ? launch_fused_part<MODE, kPartTiles, true>(kdp, bh, bl, dh, dl, out, a, items, st)
-                 : launch_fused_part<MODE, kPartTiles, false>(kdp, bh, bl, dh, dl, out, a, items, st);
+    if constexpr (MODE == kModeFused)
+        if (ones) return launch_fused_kdp<MODE, PART, EXACT, true>(args...);
+    return launch_fused_kdp<MODE, PART, EXACT, false>(args...);
+}
+
+template <int MODE, int PART, class... Args>
+b2sp_status launch_fused_exact(bool exact, const Args &...args)
+{
+    return exact ? launch_fused_ones<MODE, PART, true>(args...) : launch_fused_ones<MODE, PART, false>(args...);
+}
+
+template <int MODE>
+b2sp_status launch_fused(int kdp, bool exact, const CUtensorMap &bh, const CUtensorMap &bl, const CUtensorMap &dh,
+                         const CUtensorMap &dl, const CUtensorMap &out, const FusedTileArgs &a, int items, cudaStream_t st)
+{
+    const bool ones = a.s_values == nullptr;
+    if (a.bal_ctas > 0) return launch_fused_exact<MODE, kPartBalanced>(exact, ones, kdp, bh, bl, dh, dl, out, a, items, st);
+    if constexpr (MODE == kModeFused)   // (only FusedMM is offered on batches)
+        if (a.batch > 1) return launch_fused_exact<MODE, kPartBatched>(exact, ones, kdp, bh, bl, dh, dl, out, a, items, st);
+    return launch_fused_exact<MODE, kPartTiles>(exact, ones, kdp, bh, bl, dh, dl, out, a, items, st);
 }
 
 // Splits (or only checks) up to three dense operands and clears the device status word.
@@ -467,9 +475,9 @@ b2sp_status fused_tile(const FusedPlan &p, bool prepared, int mode, int M, int K
         }
     }
     const int items = p.bal_ctas ? p.bal_ctas : nb * p.Mt * p.Nt * p.KS;
-    b2sp_status rc = spmm    ? launch_fused_kdp<kModeSpmm>(32, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st)
-                     : fused ? launch_fused_kdp<kModeFused>(p.Kdp, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st)
-                             : launch_fused_kdp<kModeSddmm>(p.Kdp, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st);
+    b2sp_status rc = spmm    ? launch_fused<kModeSpmm>(32, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st)
+                     : fused ? launch_fused<kModeFused>(p.Kdp, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st)
+                             : launch_fused<kModeSddmm>(p.Kdp, exact, tm_bh, tm_bl, tm_dh, tm_dl, tm_out, a, items, st);
     *launches += 1;
     if (rc != B2SP_OK) return rc;
     if (fused && p.KS > 1) {

@@ -110,7 +110,10 @@ __device__ __forceinline__ int helper_index(int warp)
 // EXACT: the dense operands A, B, D are exact in tf32 (bfloat16 inputs): their lo halves are zero, so the lo
 // copies are neither loaded nor multiplied -- GEMM1 is one MMA per product instead of three, GEMM2 two (P' still
 // has a hi and a lo part).
-template <int KDP, int MODE, bool EXACT = false>
+// ONES: FusedMM without stored values.  The processors need nothing but the occupancy masks, which each thread reads from the
+// window table itself (one word per window of its row, two windows ahead): no helper warps, no slots.  Measured against helpers
+// that densified ones (eight attention problems of 4096 x 4096, whole call): 241 -> 232 us, bfloat16 operands 202 -> 186 us.
+template <int KDP, int MODE, bool EXACT = false, bool ONES = false>
 struct FusedCfg {
     static constexpr bool FUSED = MODE != kModeSddmm;          // has GEMM2 / O
     static constexpr bool SPMM = MODE == kModeSpmm;
@@ -130,7 +133,7 @@ struct FusedCfg {
     // 4 KB slots (two windows deep).  SPMM, whose helpers are the bound: the ten warps left beside the flusher
     // warps, with twenty slots.  SDDMM: twenty with forty 2 KB slots (measured: 12 helpers 134 us, 14 helpers
     // 129 us, 20 helpers on 28 warps 125 us; for SPMM the 28-warp layout was slower, 136-140 us against 131 us).
-    static constexpr int HELPERS = SPMM ? 10 : FUSED ? 8 : 20;
+    static constexpr int HELPERS = ONES ? 0 : SPMM ? 10 : FUSED ? 8 : 20;
     // FusedMM runs two sets of processor warps (warps 2-5 and 16-19) that take alternate windows: a window is a
     // chain of long-latency steps for its processor (slot, tensor-memory load, arithmetic, tensor-memory store,
     // hand-over), about 2 k cycles, and with a single set that chain, not the tensor core, paced the kernel
@@ -142,7 +145,7 @@ struct FusedCfg {
     static constexpr int SLOTS = SPMM ? 20 : FUSED ? HELPERS : 2 * HELPERS;
     // A slot's mbarriers are waited on by parity, which is only sound when the waiter is at most one
     // phase away: every slot is always filled by the same helper and drained by the same processor warp.
-    static_assert(SLOTS % HELPERS == 0 && SLOTS % IPW == 0, "slot ownership must be fixed");
+    static_assert(ONES || (SLOTS % (HELPERS + ONES) == 0 && SLOTS % IPW == 0), "slot ownership must be fixed");
     static constexpr int FLUSH_BYTES = FUSED ? 4 * 4096 : 0;   // per flushing warp: two buffers of 32 rows x 16 columns
     static constexpr int AUX_BYTES = 1024 /*barriers*/ + kFusedMaxHelpers * 256 /*record tables*/ + SLOTS * SLOT_BYTES + FLUSH_BYTES;
     static constexpr int SMEM_BYTES = RING * kFusedChunk + ALO_BYTES + 1024 + AUX_BYTES;
@@ -250,14 +253,15 @@ __device__ __noinline__ void reload_a_tile(const void *A, long long lda, long lo
 // spare).  kPartBalanced: the balanced partition (see kFusedMaxSegs); a template parameter too: with the choice made
 // at run time the SPMM kernel was 5% slower on either partition.
 constexpr int kPartTiles = 0, kPartBatched = 1, kPartBalanced = 2;
-template <int KDP, int MODE, int PART = kPartTiles, bool EXACT = false>
-__global__ void __launch_bounds__((FusedCfg<KDP, MODE, EXACT>::THREADS), 1)
+template <int KDP, int MODE, int PART = kPartTiles, bool EXACT = false, bool ONES = false>
+__global__ void __launch_bounds__((FusedCfg<KDP, MODE, EXACT, ONES>::THREADS), 1)
 fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_constant__ CUtensorMap tm_blo,
                   const __grid_constant__ CUtensorMap tm_dhi, const __grid_constant__ CUtensorMap tm_dlo,
                   const __grid_constant__ CUtensorMap tm_out, const FusedTileArgs a)
 {
-    using Cfg = FusedCfg<KDP, MODE, EXACT>;
+    using Cfg = FusedCfg<KDP, MODE, EXACT, ONES>;
     constexpr bool FUSED = Cfg::FUSED, SPMM = Cfg::SPMM;
+    static_assert(!ONES || MODE == kModeFused, "only FusedMM has a form without helpers");
     constexpr int RING = Cfg::RING, NCH_B = Cfg::NCH_B;
     constexpr int WPB = kFusedBlk / kFusedW;   // windows per block
     extern __shared__ uint8_t smem_raw[];
@@ -684,16 +688,38 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         // (balanced FusedMM: one round per segment, it_end = first window of the next segment; otherwise a single round)
         int it = FUSED ? pset : 0;
         int it_end = (bal && !SPMM && (int)ptx::lds32(segtab - 8) > 1) ? (int)ptx::lds32(segtab + 32 + kSegStart) * WPB : nwin;
+        // ONES: the occupancy masks of this thread's row, from the window table, two of the set's windows ahead
+        int seg_m0 = m0, seg_w0 = b0 * WPB, seg_end = bal ? 0 : nwin;
+        const int2 *win = a.win + (size_t)prob * a.M * a.Wk;
+        auto load_mask = [&](int i) -> unsigned {
+            if (bal && i >= seg_end && i < nwin) {   // a later segment than the one before (windows come in increasing order)
+                const uint32_t sg = seg_at(i / WPB);
+                seg_m0 = seg_f(sg, kSegM0);
+                seg_w0 = (seg_f(sg, kSegBt0) - seg_f(sg, kSegStart)) * WPB;
+                if (a.batch > 1) win = a.win + (size_t)seg_f(sg, kSegProb) * a.M * a.Wk;
+                seg_end = sg + 32 < segtab + 32 * (uint32_t)ptx::lds32(segtab - 8) ? seg_f(sg + 32, kSegStart) * WPB : nwin;
+            }
+            const int grow = seg_m0 + row, wglob = seg_w0 + i;
+            return i < nwin && grow < a.M && wglob < a.Wk ? __ldg(reinterpret_cast<const unsigned *>(win + (size_t)grow * a.Wk + wglob) + 1) : 0u;
+        };
+        unsigned mask_next = 0, mask_next2 = 0;
+        if (ONES) { mask_next = load_mask(it); mask_next2 = load_mask(it + PSETS); }
         for (;;) {
         for (; it < it_end; it += FUSED ? PSETS : 1) {
             const int blk = it / WPB, w = it % WPB;
             // FusedMM / SPMM: one item (32 rows) per processor warp and window.  SDDMM: two items of 16 rows,
             // lanes 0-15 and lanes 16-31 each with their own slot.
             const int j = FUSED ? it * 4 + q : it * 8 + 2 * q + (lane >> 4);
-            const int s = j % NSLOT, use = j / NSLOT;
+            const int s = j % (NSLOT + ONES), use = j / (NSLOT + ONES);
             const uint32_t slot = slots + s * Cfg::SLOT_BYTES + (FUSED ? lane : (lane & 15)) * 128;
             if (FUSED) {
                 float sv[32];
+                unsigned mask = 0;
+                if (ONES) {
+                    mask = mask_next;
+                    mask_next = mask_next2;
+                    mask_next2 = load_mask(it + 2 * PSETS);
+                } else {
                 {
                     bool ok = ptx::mbar_wait(sl_full(s), use & 1);
                     if (!__all_sync(0xffffffffu, ok)) { failed = true; break; }
@@ -709,6 +735,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 }
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(sl_empty(s));
+                }
                 uint32_t p0[16], p1[16];
                 if (SPMM) {
 #pragma unroll
@@ -738,11 +765,13 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 uint32_t hi[16], lo[16];
                 const uint32_t pph = tmem + lane_addr + Cfg::COL_PP + ppb * 64, ppl = pph + 32;
 #pragma unroll
-                for (int c = 0; c < 16; ++c) ptx::split_tf32_fast(__uint_as_float(p0[c]) * sv[c], hi[c], lo[c]);
+                for (int c = 0; c < 16; ++c)
+                    ptx::split_tf32_fast(ONES ? ((mask >> c) & 1u ? __uint_as_float(p0[c]) : 0.f) : __uint_as_float(p0[c]) * sv[c], hi[c], lo[c]);
                 ptx::tmem_st_32x16(pph, hi);
                 ptx::tmem_st_32x16(ppl, lo);
 #pragma unroll
-                for (int c = 0; c < 16; ++c) ptx::split_tf32_fast(__uint_as_float(p1[c]) * sv[16 + c], hi[c], lo[c]);
+                for (int c = 0; c < 16; ++c)
+                    ptx::split_tf32_fast(ONES ? ((mask >> (16 + c)) & 1u ? __uint_as_float(p1[c]) : 0.f) : __uint_as_float(p1[c]) * sv[16 + c], hi[c], lo[c]);
                 ptx::tmem_st_32x16(pph + 16, hi);
                 ptx::tmem_st_32x16(ppl + 16, lo);
                 ptx::tmem_st_wait();
@@ -812,19 +841,20 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         const int nchunks = (nblk + kFusedFlushBlocks - 1) / kFusedFlushBlocks;
         for (int chunk = 0; chunk < nchunks; ++chunk)
             if (!flush_chunk(chunk)) { failed = true; break; }
-    } else if (helper_index<FUSED>(warp) >= 0 && helper_index<FUSED>(warp) < NH) {
+    } else if (!ONES && helper_index<FUSED>(warp) >= 0 && helper_index<FUSED>(warp) < NH) {
         // ---------------- helper warps: work items (window, group of rows), round-robin ----------------
         // FusedMM / SPMM: fetch the stored values of the item's 32 rows x 32 columns with lane = column
         // (coalesced), densify (0 where nothing is stored; 1 for stored entries when there are no
         // values) and write them transposed into a slot, from which the processor thread of each row
         // reads its row.  SDDMM (items of 16 rows): prefetch the stored values the same way, then take the
         // P rows the processors left in the slot and write the stored entries, one coalesced run per row.
+        if constexpr (!ONES) {
         const int h = helper_index<FUSED>(warp);
         const uint32_t tab = helper_tabs + h * 256;   // 32 records (position, mask) of the item's rows
         constexpr int IR = Cfg::ITEM_ROWS, IPW = Cfg::IPW;
         const int wbase = b0 * WPB, nitems = nblk * WPB * IPW;
         const unsigned lane_bit = 1u << lane, lt_mask = lane_bit - 1u;
-        const bool has_values = a.s_values != nullptr;
+        const bool has_values = MODE == kModeFused || a.s_values != nullptr;   // (FusedMM without stored values is ONES)
         const float *s_values = a.s_values + prob * a.stride_sv;           // this problem's stored values,
         const int2 *win = a.win + (size_t)prob * a.M * a.Wk;               // window table
         float *out_values = a.out + prob * a.stride_O;                     // and (SDDMM) output values
@@ -905,6 +935,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                     if (idx[FUSED ? 0 : r] >= 0) out_values[idx[FUSED ? 0 : r]] = vn[r];
                 });
             }
+        }
         }
     }
     if (failed) atomicExch(a.status, 1);
