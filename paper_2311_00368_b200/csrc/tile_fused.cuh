@@ -40,9 +40,9 @@ constexpr int kFusedRows = 128;     // rows per CTA (UMMA M)
 constexpr int kFusedW = 32;         // S columns per window
 constexpr int kFusedBlk = 128;      // S columns per block (UMMA N of GEMM1)
 // FusedMM and SPMM: 20 warps = 5 per scheduler (a sixth would cut the register budget from 96 to 80 per
-// thread; measured slower).  Warp 1: MMA issue + TMEM owner; warp 9: TMA producer; warps 2-5: processors;
+// thread; measured slower).  Warp 1: MMA issue (FusedMM: GEMM1's; warp 15: GEMM2's) + TMEM owner; warp 9: TMA producer; warps 2-5: processors;
 // warps 16-19: second processor set (FusedMM) or flusher warps (SPMM); helpers among warps 0, 6-8, 10-15
-// (FusedMM: eight, none on the MMA warp's scheduler, warps 13 and 15 idle; SPMM: ten, warp 13 included).
+// (FusedMM: eight, none on the MMA warp's scheduler, warp 13 idle; SPMM: ten, warp 13 included).
 // SDDMM: 28 warps of 72 registers, see FusedCfg.
 constexpr int kFusedThreads = 640;
 constexpr int kFusedTmaWarp = 9;
@@ -54,7 +54,7 @@ constexpr int kFusedNT = 128;       // most O columns per CTA (UMMA N of GEMM2);
 // kFusedFlushBlocks blocks (192 MMAs, bias <= 4e-6), then added into the output in global memory with
 // round-to-nearest fp32 reductions and restarted from zero.
 constexpr int kFusedFlushBlocks = 4;
-constexpr int kFusedChunk = 32768;  // bytes of one pipeline chunk (hi + lo)
+constexpr int kFusedMaxSmem = 227 * 1024;   // shared memory a CTA may have
 // The balanced partition (FusedTileArgs::bal_ctas): the CTAs form groups of Nt (one CTA per column tile of O), and
 // the granules of all row tiles -- the 4-block flush granules of FusedMM / SPMM, single blocks for SDDMM -- in the order
 // (problem, row tile, granule) are dealt evenly to the groups: group c of n gets granules [c * G / n, (c + 1) * G / n)
@@ -128,7 +128,7 @@ struct FusedCfg {
     static constexpr bool DEDICATED_FLUSH = SPMM;
     static constexpr int THREADS = !FUSED ? 896 : kFusedThreads;
     static constexpr int FLUSH_WARP0 = 16;   // the flusher warps: 16-19 (SPMM: dedicated; FusedMM: the second processor set)
-    static constexpr int RING = FUSED ? 3 : 4;   // TMA chunks in flight (32 KB each)
+    static constexpr int CHUNK = EXACT ? 16384 : 32768;   // bytes of one pipeline chunk (hi + lo)
     // FusedMM is bound by the tensor pipe and its helpers are mostly idle: eight of them, with eight
     // 4 KB slots (two windows deep).  SPMM, whose helpers are the bound: the ten warps left beside the flusher
     // warps, with twenty slots.  SDDMM: twenty with forty 2 KB slots (measured: 12 helpers 134 us, 14 helpers
@@ -139,6 +139,8 @@ struct FusedCfg {
     // hand-over), about 2 k cycles, and with a single set that chain, not the tensor core, paced the kernel
     // wherever a window holds less than 2 k cycles of MMAs.  The second set (odd windows) also does the flushes.
     static constexpr int PSETS = (FUSED && !SPMM) ? 2 : 1;
+    static constexpr bool TWO_ISSUERS = FUSED && !SPMM;
+    static constexpr int G2_WARP = TWO_ISSUERS ? 15 : 1;      // the warp that issues GEMM2
     static constexpr int ITEM_ROWS = FUSED ? 32 : 16;           // rows of a helper's work item
     static constexpr int IPW = kFusedRows / ITEM_ROWS;         // items per window
     static constexpr int SLOT_BYTES = ITEM_ROWS * 128;
@@ -146,9 +148,15 @@ struct FusedCfg {
     // A slot's mbarriers are waited on by parity, which is only sound when the waiter is at most one
     // phase away: every slot is always filled by the same helper and drained by the same processor warp.
     static_assert(ONES || (SLOTS % (HELPERS + ONES) == 0 && SLOTS % IPW == 0), "slot ownership must be fixed");
-    static constexpr int FLUSH_BYTES = FUSED ? 4 * 4096 : 0;   // per flushing warp: two buffers of 32 rows x 16 columns
+    static constexpr int FLUSH_BUFS = !FUSED ? 0 : ONES || SPMM || EXACT ? 4 : 3;   // per flushing warp: buffers of 32 rows x 16 columns
+    static constexpr int FLUSH_BYTES = 4 * FLUSH_BUFS * 2048;
     static constexpr int AUX_BYTES = 1024 /*barriers*/ + kFusedMaxHelpers * 256 /*record tables*/ + SLOTS * SLOT_BYTES + FLUSH_BYTES;
-    static constexpr int SMEM_BYTES = RING * kFusedChunk + ALO_BYTES + 1024 + AUX_BYTES;
+    // TMA chunks in flight: what the shared memory holds beside the rest.  (ONES with lo halves: three.  With four or five, GEMM1 of
+    // the next block runs ahead of GEMM2 and the eight attention problems take 219 instead of 211 us.)
+    static constexpr int RING_FIT = (kFusedMaxSmem - ALO_BYTES - 1024 - AUX_BYTES) / CHUNK;
+    static constexpr int RING_MOST = ONES && !EXACT ? 3 : 8;
+    static constexpr int RING = RING_FIT < RING_MOST ? RING_FIT : RING_MOST;
+    static constexpr int SMEM_BYTES = RING * CHUNK + ALO_BYTES + 1024 + AUX_BYTES;
     // tensor-memory columns
     // SPMM has tensor memory to spare: two O accumulators, so that the tensor core works on the next
     // chunk of blocks while the previous partial sum is flushed.
@@ -262,16 +270,19 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
     using Cfg = FusedCfg<KDP, MODE, EXACT, ONES>;
     constexpr bool FUSED = Cfg::FUSED, SPMM = Cfg::SPMM;
     static_assert(!ONES || MODE == kModeFused, "only FusedMM has a form without helpers");
-    constexpr int RING = Cfg::RING, NCH_B = Cfg::NCH_B;
+    constexpr int RING = Cfg::RING, CHUNK = Cfg::CHUNK, NCH_B = Cfg::NCH_B;
     constexpr int WPB = kFusedBlk / kFusedW;   // windows per block
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - ptx::smem_u32(smem_raw));
-    const uint32_t ring = smem_base;                               // RING chunks of 32 KB
-    const uint32_t alo_smem = smem_base + RING * kFusedChunk;      // FusedMM: A_lo, K-major, 16 KB per 32 k
+    const uint32_t ring = smem_base;                               // RING chunks
+    const uint32_t alo_smem = smem_base + RING * CHUNK;      // FusedMM: A_lo, K-major, 16 KB per 32 k
     const uint32_t aux = alo_smem + Cfg::ALO_BYTES;
     auto full = [&](int s) { return aux + 8u * s; };
     auto empty = [&](int s) { return aux + 8u * (RING + s); };
+    // FusedMM: B and D chunks share the ring but complete on barriers of their own: each has one waiting thread, which has
+    // always seen the previous phase (waits by parity need that)
+    auto full_d = [&](int s) { return Cfg::TWO_ISSUERS ? aux + 512 + 8u * s : full(s); };
     auto p_full = [&](int b) { return aux + 8u * (2 * RING + b); };
     auto p_free = [&](int b) { return aux + 8u * (2 * RING + 2 + b); };
     auto pp_full = [&](int b) { return aux + 8u * (2 * RING + 4 + b); };
@@ -337,7 +348,11 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
     auto seg_f = [&](uint32_t rec, uint32_t field) -> int { return (int)ptx::lds32(rec + field); };
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < RING; ++s) { ptx::mbar_init(full(s), 1); ptx::mbar_init(empty(s), 1); }
+        for (int s = 0; s < RING; ++s) {
+            ptx::mbar_init(full(s), 1);
+            ptx::mbar_init(empty(s), 1);
+            if (Cfg::TWO_ISSUERS) ptx::mbar_init(full_d(s), 1);
+        }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(p_full(b), 1);
             ptx::mbar_init(p_free(b), FUSED ? 4 * Cfg::PSETS : 4);
@@ -411,23 +426,24 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         bool ok = ptx::mbar_wait(o_full(ob), (chunk / NOB) & 1);
         if (!__all_sync(0xffffffffu, ok)) return false;
         ptx::tc_fence_after_sync();
-        // 16 columns at a time go through shared memory (per warp two buffers of 32 rows x 16
+        // 16 columns at a time go through shared memory (per warp a few buffers of 32 rows x 16
         // columns, 64-byte swizzle: 16-byte piece j of row r at piece j ^ ((r >> 1) & 3)).  From
         // there one TMA store (first partial sum) or fp32 add-reduction per buffer moves whole
         // 64-byte row pieces; rows and columns outside the output are clipped by TMA.  O is free
         // for the tensor core again as soon as its last columns have been read.
-        const uint32_t stage = flush_stage + (uint32_t)q * 4096;
+        const uint32_t stage = flush_stage + (uint32_t)q * (Cfg::FLUSH_BUFS * 2048);
         if (a.out_tma) {
             if (ptx::elect_one()) ptx::bulk_wait<0>();   // the previous flush's reductions are complete (order of the sums)
             __syncwarp();
             // one K split: the output itself, problem = third coordinate; several: the slabs, stacked
             const int y = (a.KS == 1 ? 0 : (prob * a.KS + ks) * a.slab_rows) + m0 + q * 32;
             const int z = a.KS == 1 ? prob : 0;
+            constexpr int NBUF = Cfg::FLUSH_BUFS ? Cfg::FLUSH_BUFS : 1;
 #pragma unroll 1
             for (int c = 0; c < a.NT / 16; ++c) {
-                const uint32_t buf = stage + (uint32_t)(c & 1) * 2048;
-                if (c >= 2) {
-                    if (ptx::elect_one()) ptx::bulk_wait_read<1>();   // the buffer's previous contents have been read
+                const uint32_t buf = stage + (uint32_t)(c % NBUF) * 2048;
+                if (c >= NBUF) {
+                    if (ptx::elect_one()) ptx::bulk_wait_read<NBUF - 1>();   // the buffer's previous contents have been read
                     __syncwarp();
                 }
                 uint32_t r[16];
@@ -511,17 +527,23 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         if (ptx::elect_one()) {
             if (!SPMM) { ptx::tma_prefetch_desc(&tm_bhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_blo); }
             if (FUSED) { ptx::tma_prefetch_desc(&tm_dhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_dlo); }
-            // Chunk order = the order the MMA thread consumes them: B(0); then per block b:
+            // Chunk order = the order the MMA issuers consume them: B(0); then per block b:
             // D(b,0) D(b,1) | B(b+1) | D(b,2) D(b,3)   (SDDMM: B chunks only; last block of a chunk: B(b+1) last).
-            int c = 0;
+            int c = 0, slot = 0;
+            uint32_t empty_phase = 1;   // parity of the slot's previous use
+            uint32_t phase_b = 0, phase_d = 0, last_d = 0;   // per slot: parity of its next B chunk and D chunk, whether a D chunk is its last one
             // first row of the CTA's block 0 in the stacked operand copies, column tile, and (balanced partition) the
             // block at which the next segment begins
             int seg_col0 = krow0 + b0 * kFusedBlk, ntile = nt, seg_end = bal ? 0 : nblk;
             auto put = [&](bool is_b, int blk, int i) -> bool {
-                const int s = c % RING;
-                if (c >= RING && !ptx::mbar_wait(empty(s), ((c / RING) - 1) & 1)) return false;
-                if (c == a.debug_drop_chunk) { ++c; return true; }   // (test hook: nobody will ever complete this chunk's barrier)
-                const uint32_t dst = ring + s * kFusedChunk;
+                if (c >= RING && !ptx::mbar_wait(empty(slot), empty_phase)) return false;
+                const uint32_t bit = 1u << slot;
+                if (is_b) { phase_b ^= bit; last_d &= ~bit; }
+                else { phase_d ^= bit; last_d |= bit; }
+                const int s = slot;
+                if (++slot == RING) { slot = 0; empty_phase ^= 1; }
+                if (c++ == a.debug_drop_chunk) return true;   // (test hook: nobody will ever complete this chunk's barrier)
+                const uint32_t dst = ring + s * CHUNK;
                 if (bal && blk >= seg_end) {   // a later segment than the one before (the blocks come in increasing order)
                     const uint32_t sg = seg_at(blk);
                     seg_col0 = seg_f(sg, kSegProb) * a.Kp + (seg_f(sg, kSegBt0) - seg_f(sg, kSegStart)) * kFusedBlk;
@@ -529,36 +551,90 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                     seg_end = sg + 32 < segtab + 32 * (uint32_t)ptx::lds32(segtab - 8) ? seg_f(sg + 32, kSegStart) : nblk;
                 }
                 const int col0 = seg_col0 + blk * kFusedBlk;
-                ptx::mbar_arrive_expect_tx(full(s), (is_b ? kFusedChunk : 2 * kFusedW * a.NT * 4) / (EXACT ? 2 : 1));   // hi (+ lo)
+                const uint32_t bar = is_b ? full(s) : full_d(s);
+                ptx::mbar_arrive_expect_tx(bar, is_b ? CHUNK : (EXACT ? 1 : 2) * kFusedW * a.NT * 4);   // hi (+ lo)
                 if (is_b) {   // B rows col0..col0+127, k group i
-                    ptx::tma_load_3d(dst, &tm_bhi, full(s), 0, col0, i);
-                    if (!EXACT) ptx::tma_load_3d(dst + kFusedChunk / 2, &tm_blo, full(s), 0, col0, i);
+                    ptx::tma_load_3d(dst, &tm_bhi, bar, 0, col0, i);
+                    if (!EXACT) ptx::tma_load_3d(dst + CHUNK / 2, &tm_blo, bar, 0, col0, i);
                 } else {      // D rows of window i of the block
                     const int krow = col0 + i * kFusedW;
-                    ptx::tma_load_3d(dst, &tm_dhi, full(s), 0, krow, ntile * (a.NT / 32));
+                    ptx::tma_load_3d(dst, &tm_dhi, bar, 0, krow, ntile * (a.NT / 32));
                     // (64-column O tiles: the lo copy sits right behind the 8 KB hi copy, so that [hi | lo] is one
                     // MN-major operand of 128 columns, see GEMM2)
-                    if (!EXACT) ptx::tma_load_3d(dst + (a.NT == 64 ? kFusedW * 64 * 4 : kFusedChunk / 2), &tm_dlo, full(s), 0, krow, ntile * (a.NT / 32));
+                    if (!EXACT) ptx::tma_load_3d(dst + (a.NT == 64 ? kFusedW * 64 * 4 : CHUNK / 2), &tm_dlo, bar, 0, krow, ntile * (a.NT / 32));
                 }
-                ++c;
                 return true;
             };
             for (int i = 0; i < NCH_B && nblk > 0 && !failed; ++i) failed = !put(true, 0, i);
             for (int b = 0; b < nblk && !failed; ++b) {
-                // (FusedMM: at the end of a chunk of blocks GEMM1 of the next block comes last, see the MMA thread)
+                // (FusedMM: at the end of a chunk of blocks GEMM1 of the next block comes last, see the MMA issuers)
                 const bool late_b = FUSED && b % kFusedFlushBlocks == kFusedFlushBlocks - 1;
                 if (FUSED) for (int w = 0; w < 2 && !failed; ++w) failed = !put(false, b, w);
                 if (!SPMM && b + 1 < nblk && !late_b) for (int i = 0; i < NCH_B && !failed; ++i) failed = !put(true, b + 1, i);
                 if (FUSED) for (int w = 2; w < WPB && !failed; ++w) failed = !put(false, b, w);
                 if (!SPMM && b + 1 < nblk && late_b) for (int i = 0; i < NCH_B && !failed; ++i) failed = !put(true, b + 1, i);
             }
-            if (failed)
-                for (int j = c > RING ? c - RING : 0; j < c; ++j) ptx::mbar_wait(full(j % RING), (j / RING) & 1);
+            if (failed)   // (its own copies in flight are waited for)
+                for (int j = 0; j < RING && j < c; ++j) {
+                    const bool d = Cfg::TWO_ISSUERS && ((last_d >> j) & 1u);
+                    ptx::mbar_wait(d ? full_d(j) : full(j), (((Cfg::TWO_ISSUERS ? (d ? phase_d : phase_b) : phase_b ^ phase_d) >> j) & 1u) ^ 1u);
+                }
         }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
+    } else if (!SPMM && warp == 1) {
+        // ---------------- GEMM1 issuer: P = A_tile * B_block^T ----------------
+        // GEMM1 and GEMM2 (below) have an issuing thread each.  What an issuing thread does for one chunk beside its MMAs -- barrier
+        // checks, commits, bookkeeping, at 6 or more cycles an instruction -- takes it about as long as the tensor core needs for
+        // the chunk: one thread for both was what paced the kernel, with 97% of the barriers it asked for long complete and 62% of
+        // its time spent between them even with MMAs cut to a quarter.  Whole calls, one thread -> two and descriptors in halves:
+        // eight attention problems 233 -> 211 us, bfloat16 operands (with a ring of eight chunks, not three) 186 -> 165 us,
+        // power-law 8192 x 8192 x 128 at 30% 189 -> 181 us.
         if (ptx::elect_one()) {
+            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, 16, 1024, ptx::kLayoutSw128) >> 32);
             constexpr uint32_t idesc1 = ptx::idesc_tf32(kFusedRows, kFusedBlk, false, false);
+            int slot = 0;
+            uint32_t phase = 0;   // per slot: parity of its next B chunk
+            // balanced partition: the next segment whose A tile GEMM1 will need, and its first block
+            int a_seg = 1, a_next = (bal && (int)ptx::lds32(segtab - 8) > 1) ? (int)ptx::lds32(segtab + 32 + kSegStart) : -1;
+            auto late = [](int b) { return FUSED && b % kFusedFlushBlocks == kFusedFlushBlocks - 1; };
+            for (int b = 0; b < nblk && !failed; ++b) {
+                const int pb = FUSED ? 0 : (b & 1), puse = FUSED ? b : (b >> 1);
+                if (FUSED && b > 0) {   // the D chunks between the previous block's B chunks and this one's
+                    slot += (b > 1 && !late(b - 2) ? 2 : 0) + (late(b - 1) ? 4 : 2);
+                    while (slot >= RING) slot -= RING;
+                }
+                if (puse > 0 && !ptx::mbar_wait(p_free(pb), (puse - 1) & 1)) { failed = true; break; }   // P drained?
+                if (bal && b == a_next) {
+                    // first block of a new segment: the processors have put the next row tile of A in place
+                    if (!ptx::mbar_wait(a_ready, (a_seg - 1) & 1)) { failed = true; break; }
+                    ++a_seg;
+                    a_next = a_seg < (int)ptx::lds32(segtab - 8) ? (int)ptx::lds32(segtab + a_seg * 32 + kSegStart) : -1;
+                }
+                ptx::tc_fence_after_sync();
+                const uint32_t pacc = tmem + Cfg::COL_P + pb * kFusedBlk;
+                for (int i = 0; i < NCH_B; ++i) {
+                    if (!ptx::mbar_wait(full(slot), (phase >> slot) & 1u)) { failed = true; break; }
+                    const uint32_t b_hi = (uint32_t)ptx::smem_desc(ring + slot * CHUNK, 16, 1024, ptx::kLayoutSw128), b_lo = b_hi + (CHUNK / 2 >> 4);
+                    const uint32_t a_lo = (uint32_t)ptx::smem_desc(alo_smem + i * (kFusedRows * 128), 16, 1024, ptx::kLayoutSw128);
+                    const uint32_t acol = tmem + Cfg::COL_AHI + i * 32;
+#pragma unroll
+                    for (int k8 = 0; k8 < 4; ++k8) {
+                        ptx::mma_tf32_ts(pacc, acol + k8 * 8, b_hi + k8 * 2, desc_up, idesc1, (i | k8) != 0);
+                        if (EXACT) continue;   // A and B exact in tf32: no lo terms
+                        ptx::mma_tf32_ts(pacc, acol + k8 * 8, b_lo + k8 * 2, desc_up, idesc1, 1);
+                        if (FUSED) ptx::mma_tf32_ss(pacc, a_lo + k8 * 2, desc_up, b_hi + k8 * 2, desc_up, idesc1, 1);
+                        else ptx::mma_tf32_ts(pacc, acol + (Cfg::COL_ALO - Cfg::COL_AHI) + k8 * 8, b_hi + k8 * 2, desc_up, idesc1, 1);
+                    }
+                    ptx::mma_commit(empty(slot));
+                    phase ^= 1u << slot;
+                    if (++slot == RING) slot = 0;
+                }
+                ptx::mma_commit(p_full(pb));
+            }
+        }
+    } else if (FUSED && warp == Cfg::G2_WARP) {
+        // ---------------- GEMM2 issuer: O += P'_window * D_window ----------------
+        if (ptx::elect_one()) {
+            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, kFusedW * 128, 512, ptx::kLayoutSw128Base32) >> 32);
             const uint32_t idesc2 = a.NT == 64 ? ptx::idesc_tf32(kFusedRows, 64, false, true) : ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
             constexpr uint32_t idesc2_cat = ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
             // 64-column O tiles (N <= 64): a 64-column MMA would leave half of the tensor core's width unused (it takes 46
@@ -566,114 +642,52 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             // columns 0-63 and 64-127 of the accumulator, P'_lo by D_hi in a 64-column one: two MMAs per K step instead
             // of three; the flush adds the two halves.
             const bool cat = !EXACT && a.NT == 64;
-            int c = 0, ppu = 0;   // chunk counter, P' buffer uses so far
-            // The chunk after the one whose MMAs are being issued is asked for halfway through them: the tensor pipe has
-            // about three MMAs queued then, which hide one barrier check (~100 cycles) but not two in a row.  (Not with
-            // bfloat16 operands: a chunk is a third of the MMAs there, and asking early meant waiting for data: +4%.)
-            const int nchunk = nblk * (NCH_B + Cfg::NCH_D);
-            int arrived = 0;   // chunks known to be in shared memory
-            auto chunk_arrived = [&](int want) -> bool {
-                if (want < arrived || want >= nchunk) return true;
-                arrived = want + 1;
-                return ptx::mbar_wait(full(want % RING), (want / RING) & 1);
+            int slot = NCH_B % RING, ppb = 0;
+            uint32_t phase = 0, pp_phase = 0;   // per slot: parity of its next D chunk; parity of the P' buffers' next use
+            auto skip_b = [&] {   // the next block's B chunks
+                slot += NCH_B;
+                while (slot >= RING) slot -= RING;
             };
-            // balanced partition: the next segment whose A tile GEMM1 will need, and its first block
-            int a_seg = 1, a_next = (bal && !SPMM && (int)ptx::lds32(segtab - 8) > 1) ? (int)ptx::lds32(segtab + 32 + kSegStart) : -1;
-            auto gemm1 = [&](int b) -> bool {   // P = A_tile * B_block^T over NCH_B chunks
-                const int pb = FUSED ? 0 : (b & 1);
-                const int puse = FUSED ? b : (b >> 1);
-                if (puse > 0 && !ptx::mbar_wait(p_free(pb), (puse - 1) & 1)) return false;   // P drained?
-                if (bal && !SPMM && b == a_next) {
-                    // first block of a new segment: the processors have put the next row tile of A in place
-                    if (!ptx::mbar_wait(a_ready, (a_seg - 1) & 1)) return false;
+            for (int b = 0; b < nblk && !failed; ++b) {
+                const int ch = b / kFusedFlushBlocks, b_in = b % kFusedFlushBlocks;
+                // O restarts from zero every kFusedFlushBlocks blocks, once the partial sum before (chunk ch reuses the accumulator
+                // of chunk ch - NOB) has been taken out of tensor memory
+                if (b_in == 0 && ch >= NOB && !ptx::mbar_wait(o_free(ch % NOB), (ch / NOB - 1) & 1)) { failed = true; break; }
+                const uint32_t oacc = tmem + Cfg::COL_O + (ch % NOB) * kFusedNT;
+                const bool late_b = b_in == kFusedFlushBlocks - 1;
+                for (int w = 0; w < WPB; ++w) {
+                    if (!ptx::mbar_wait(pp_full(ppb), pp_phase) || !ptx::mbar_wait(full_d(slot), (phase >> slot) & 1u)) { failed = true; break; }
                     ptx::tc_fence_after_sync();
-                    ++a_seg;
-                    a_next = a_seg < (int)ptx::lds32(segtab - 8) ? (int)ptx::lds32(segtab + a_seg * 32 + kSegStart) : -1;
-                }
-                const uint32_t pacc = tmem + Cfg::COL_P + pb * kFusedBlk;
-                for (int i = 0; i < NCH_B; ++i, ++c) {
-                    const int s = c % RING;
-                    if (!chunk_arrived(c)) return false;
-                    ptx::tc_fence_after_sync();
-                    const uint32_t b_hi = ring + s * kFusedChunk, b_lo = b_hi + kFusedChunk / 2;
+                    // D window: MN-major tf32 (32-byte-atom swizzle): column groups 4 KB apart, 4-row K groups 512 B apart,
+                    // +1 KB per K step of 8 rows.  (Two copies of the loop: a test inside it costs the issuing thread.)
+                    const uint32_t d_hi = (uint32_t)ptx::smem_desc(ring + slot * CHUNK, kFusedW * 128, 512, ptx::kLayoutSw128Base32), d_lo = d_hi + (CHUNK / 2 >> 4);
+                    const uint32_t pph = tmem + Cfg::COL_PP + ppb * 64, ppl = pph + 32;
+                    const uint32_t first = (b_in | w) != 0;   // 0: this MMA starts a new partial sum
+                    if (cat) {
 #pragma unroll
-                    for (int k8 = 0; k8 < 4; ++k8) {
-                        const uint64_t dbh = ptx::smem_desc(b_hi + k8 * 32, 16, 1024, ptx::kLayoutSw128);
-                        const uint64_t dbl = ptx::smem_desc(b_lo + k8 * 32, 16, 1024, ptx::kLayoutSw128);
-                        const uint32_t acol = i * 32 + k8 * 8;
-                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
-                        ptx::mma_tf32_ts(pacc, tmem + Cfg::COL_AHI + acol, dbh, idesc1, (i | k8) != 0);
-                        if (EXACT) continue;   // A and B exact in tf32: no lo terms
-                        ptx::mma_tf32_ts(pacc, tmem + Cfg::COL_AHI + acol, dbl, idesc1, 1);
-                        if (FUSED) {
-                            const uint64_t dal = ptx::smem_desc(alo_smem + i * (kFusedRows * 128) + k8 * 32, 16, 1024, ptx::kLayoutSw128);
-                            ptx::mma_tf32_ss(pacc, dal, dbh, idesc1, 1);
-                        } else {
-                            ptx::mma_tf32_ts(pacc, tmem + Cfg::COL_ALO + acol, dbh, idesc1, 1);
+                        for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
+                            ptx::mma_tf32_ts(oacc, pph + k8 * 8, d_hi + k8 * 64, desc_up, idesc2_cat, k8 == 0 ? first : 1u);
+                            ptx::mma_tf32_ts(oacc, ppl + k8 * 8, d_hi + k8 * 64, desc_up, idesc2, 1);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
+                            ptx::mma_tf32_ts(oacc, pph + k8 * 8, d_hi + k8 * 64, desc_up, idesc2, k8 == 0 ? first : 1u);
+                            ptx::mma_tf32_ts(oacc, ppl + k8 * 8, d_hi + k8 * 64, desc_up, idesc2, 1);
+                            if (!EXACT) ptx::mma_tf32_ts(oacc, pph + k8 * 8, d_lo + k8 * 64, desc_up, idesc2, 1);
                         }
                     }
-                    ptx::mma_commit(empty(s));
+                    ptx::mma_commit(pp_free(ppb));
+                    ptx::mma_commit(empty(slot));
+                    phase ^= 1u << slot;
+                    if (++slot == RING) slot = 0;
+                    pp_phase ^= ppb;
+                    ppb ^= 1;
+                    if (!SPMM && w == 1 && !late_b && b + 1 < nblk) skip_b();
                 }
-                ptx::mma_commit(p_full(pb));
-                return true;
-            };
-            auto gemm2 = [&](int b, int w) -> bool {   // O += P'_window * D_window
-                const int s = c % RING, ppb = ppu & 1;
-                if (!ptx::mbar_wait(pp_full(ppb), (ppu >> 1) & 1)) return false;
-                if (!chunk_arrived(c)) return false;
-                ptx::tc_fence_after_sync();
-                const uint32_t d_hi = ring + s * kFusedChunk, d_lo = d_hi + kFusedChunk / 2;
-                const uint32_t pph = tmem + Cfg::COL_PP + ppb * 64, ppl = pph + 32;
-                const uint32_t oacc = tmem + Cfg::COL_O + ((b / kFusedFlushBlocks) % NOB) * kFusedNT;
-                // D window: MN-major tf32 (32-byte-atom swizzle): column groups 4 KB apart, 4-row K groups 512 B apart,
-                // +1 KB per K step of 8 rows.  (Two copies of the loop: a test inside it costs the issuing thread, whose
-                // instruction stream paces the tensor pipe, several percent.)
-                const uint32_t first = ((b % kFusedFlushBlocks) | w) != 0;   // 0: this MMA starts a new partial sum
-                if (cat) {
-#pragma unroll
-                    for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
-                        const uint64_t ddh = ptx::smem_desc(d_hi + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
-                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
-                        ptx::mma_tf32_ts(oacc, pph + k8 * 8, ddh, idesc2_cat, k8 == 0 ? first : 1u);
-                        ptx::mma_tf32_ts(oacc, ppl + k8 * 8, ddh, idesc2, 1);
-                    }
-                } else {
-#pragma unroll
-                    for (int k8 = 0; k8 < kFusedW / 8; ++k8) {
-                        const uint64_t ddh = ptx::smem_desc(d_hi + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
-                        if (!EXACT && k8 == 2 && !chunk_arrived(c + 1)) return false;
-                        const uint64_t ddl = ptx::smem_desc(d_lo + k8 * 1024, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
-                        ptx::mma_tf32_ts(oacc, pph + k8 * 8, ddh, idesc2, k8 == 0 ? first : 1u);
-                        ptx::mma_tf32_ts(oacc, ppl + k8 * 8, ddh, idesc2, 1);
-                        if (!EXACT) ptx::mma_tf32_ts(oacc, pph + k8 * 8, ddl, idesc2, 1);
-                    }
-                }
-                ptx::mma_commit(pp_free(ppb));
-                ptx::mma_commit(empty(s));
-                ++c;
-                ++ppu;
-                return true;
-            };
-            // GEMM1 of block b+1 is issued between the second and third GEMM2 of block b: by then the
-            // element-wise warps have read all of P(b), and the tensor pipe has work while they
-            // process the last two windows of block b.
-            if (!SPMM && nblk > 0 && !gemm1(0)) failed = true;
-            for (int b = 0; b < nblk && !failed; ++b) {
-                // O restarts from zero every kFusedFlushBlocks blocks, once the processors have taken the
-                // previous partial sum out of tensor memory
-                if (FUSED && b % kFusedFlushBlocks == 0 && b / kFusedFlushBlocks >= NOB) {
-                    const int ch = b / kFusedFlushBlocks;   // chunk ch reuses the accumulator of chunk ch - NOB
-                    failed = !ptx::mbar_wait(o_free(ch % NOB), (ch / NOB - 1) & 1);
-                }
-                // At the end of a chunk GEMM1 of the next block is issued after the chunk's last GEMM2, so that
-                // the tensor core works on it while the processors take O out of tensor memory.
-                const bool late_b = FUSED && b % kFusedFlushBlocks == kFusedFlushBlocks - 1;
-                if (FUSED) for (int w = 0; w < 2 && !failed; ++w) failed = !gemm2(b, w);
-                if (!SPMM && b + 1 < nblk && !late_b && !failed) failed = !gemm1(b + 1);
-                if (FUSED) for (int w = 2; w < WPB && !failed; ++w) failed = !gemm2(b, w);
-                if (FUSED && !failed && (late_b || b == nblk - 1))
-                    ptx::mma_commit(o_full((b / kFusedFlushBlocks) % NOB));
-                if (!SPMM && b + 1 < nblk && late_b && !failed) failed = !gemm1(b + 1);
+                if (failed) break;
+                if (late_b || b == nblk - 1) ptx::mma_commit(o_full(ch % NOB));
+                if (!SPMM && late_b && b + 1 < nblk) skip_b();
             }
         }
     } else if ((warp >= 2 && warp < 6) || (Cfg::PSETS == 2 && warp >= 16)) {
