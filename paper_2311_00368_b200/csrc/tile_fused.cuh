@@ -140,6 +140,10 @@ struct FusedCfg {
     // wherever a window holds less than 2 k cycles of MMAs.  The second set (odd windows) also does the flushes.
     static constexpr int PSETS = (FUSED && !SPMM) ? 2 : 1;
     static constexpr bool TWO_ISSUERS = FUSED && !SPMM;
+    // B of the next block after all four windows of D at the end of a chunk of blocks (the tensor core works on GEMM1 while O is flushed)
+    // instead of after two of them.  Not with operands exact in tf32, whose GEMM1 is too short to cover the flush and whose ring holds
+    // both (eight attention problems: 162 us with the same order throughout, 165 with this one; fp32 operands 221 and 211).
+    static constexpr bool LATE_B = TWO_ISSUERS && !EXACT;
     static constexpr int G2_WARP = TWO_ISSUERS ? 15 : 1;      // the warp that issues GEMM2
     static constexpr int ITEM_ROWS = FUSED ? 32 : 16;           // rows of a helper's work item
     static constexpr int IPW = kFusedRows / ITEM_ROWS;         // items per window
@@ -532,9 +536,9 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             int c = 0, slot = 0;
             uint32_t empty_phase = 1;   // parity of the slot's previous use
             uint32_t phase_b = 0, phase_d = 0, last_d = 0;   // per slot: parity of its next B chunk and D chunk, whether a D chunk is its last one
-            // first row of the CTA's block 0 in the stacked operand copies, column tile, and (balanced partition) the
-            // block at which the next segment begins
-            int seg_col0 = krow0 + b0 * kFusedBlk, ntile = nt, seg_end = bal ? 0 : nblk;
+            // for B and for D (whose chunks may be a segment apart): first row of the CTA's block 0 in the stacked operand copies, column
+            // tile, and (balanced partition) the block at which the next segment begins
+            struct { int col0, ntile, end; } seg_b = {krow0 + b0 * kFusedBlk, nt, bal ? 0 : nblk}, seg_d = seg_b;
             auto put = [&](bool is_b, int blk, int i) -> bool {
                 if (c >= RING && !ptx::mbar_wait(empty(slot), empty_phase)) return false;
                 const uint32_t bit = 1u << slot;
@@ -544,13 +548,14 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 if (++slot == RING) { slot = 0; empty_phase ^= 1; }
                 if (c++ == a.debug_drop_chunk) return true;   // (test hook: nobody will ever complete this chunk's barrier)
                 const uint32_t dst = ring + s * CHUNK;
-                if (bal && blk >= seg_end) {   // a later segment than the one before (the blocks come in increasing order)
+                auto &seg = is_b ? seg_b : seg_d;
+                if (bal && blk >= seg.end) {   // a later segment than the one before (the blocks come in increasing order)
                     const uint32_t sg = seg_at(blk);
-                    seg_col0 = seg_f(sg, kSegProb) * a.Kp + (seg_f(sg, kSegBt0) - seg_f(sg, kSegStart)) * kFusedBlk;
-                    ntile = seg_f(sg, kSegNt);
-                    seg_end = sg + 32 < segtab + 32 * (uint32_t)ptx::lds32(segtab - 8) ? seg_f(sg + 32, kSegStart) : nblk;
+                    seg.col0 = seg_f(sg, kSegProb) * a.Kp + (seg_f(sg, kSegBt0) - seg_f(sg, kSegStart)) * kFusedBlk;
+                    seg.ntile = seg_f(sg, kSegNt);
+                    seg.end = sg + 32 < segtab + 32 * (uint32_t)ptx::lds32(segtab - 8) ? seg_f(sg + 32, kSegStart) : nblk;
                 }
-                const int col0 = seg_col0 + blk * kFusedBlk;
+                const int col0 = seg.col0 + blk * kFusedBlk;
                 const uint32_t bar = is_b ? full(s) : full_d(s);
                 ptx::mbar_arrive_expect_tx(bar, is_b ? CHUNK : (EXACT ? 1 : 2) * kFusedW * a.NT * 4);   // hi (+ lo)
                 if (is_b) {   // B rows col0..col0+127, k group i
@@ -558,17 +563,17 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                     if (!EXACT) ptx::tma_load_3d(dst + CHUNK / 2, &tm_blo, bar, 0, col0, i);
                 } else {      // D rows of window i of the block
                     const int krow = col0 + i * kFusedW;
-                    ptx::tma_load_3d(dst, &tm_dhi, bar, 0, krow, ntile * (a.NT / 32));
+                    ptx::tma_load_3d(dst, &tm_dhi, bar, 0, krow, seg.ntile * (a.NT / 32));
                     // (64-column O tiles: the lo copy sits right behind the 8 KB hi copy, so that [hi | lo] is one
                     // MN-major operand of 128 columns, see GEMM2)
-                    if (!EXACT) ptx::tma_load_3d(dst + (a.NT == 64 ? kFusedW * 64 * 4 : CHUNK / 2), &tm_dlo, bar, 0, krow, ntile * (a.NT / 32));
+                    if (!EXACT) ptx::tma_load_3d(dst + (a.NT == 64 ? kFusedW * 64 * 4 : CHUNK / 2), &tm_dlo, bar, 0, krow, seg.ntile * (a.NT / 32));
                 }
                 return true;
             };
             for (int i = 0; i < NCH_B && nblk > 0 && !failed; ++i) failed = !put(true, 0, i);
             for (int b = 0; b < nblk && !failed; ++b) {
                 // (FusedMM: at the end of a chunk of blocks GEMM1 of the next block comes last, see the MMA issuers)
-                const bool late_b = FUSED && b % kFusedFlushBlocks == kFusedFlushBlocks - 1;
+                const bool late_b = Cfg::LATE_B && b % kFusedFlushBlocks == kFusedFlushBlocks - 1;
                 if (FUSED) for (int w = 0; w < 2 && !failed; ++w) failed = !put(false, b, w);
                 if (!SPMM && b + 1 < nblk && !late_b) for (int i = 0; i < NCH_B && !failed; ++i) failed = !put(true, b + 1, i);
                 if (FUSED) for (int w = 2; w < WPB && !failed; ++w) failed = !put(false, b, w);
@@ -595,7 +600,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             uint32_t phase = 0;   // per slot: parity of its next B chunk
             // balanced partition: the next segment whose A tile GEMM1 will need, and its first block
             int a_seg = 1, a_next = (bal && (int)ptx::lds32(segtab - 8) > 1) ? (int)ptx::lds32(segtab + 32 + kSegStart) : -1;
-            auto late = [](int b) { return FUSED && b % kFusedFlushBlocks == kFusedFlushBlocks - 1; };
+            auto late = [](int b) { return Cfg::LATE_B && b % kFusedFlushBlocks == kFusedFlushBlocks - 1; };
             for (int b = 0; b < nblk && !failed; ++b) {
                 const int pb = FUSED ? 0 : (b & 1), puse = FUSED ? b : (b >> 1);
                 if (FUSED && b > 0) {   // the D chunks between the previous block's B chunks and this one's
@@ -654,7 +659,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 // of chunk ch - NOB) has been taken out of tensor memory
                 if (b_in == 0 && ch >= NOB && !ptx::mbar_wait(o_free(ch % NOB), (ch / NOB - 1) & 1)) { failed = true; break; }
                 const uint32_t oacc = tmem + Cfg::COL_O + (ch % NOB) * kFusedNT;
-                const bool late_b = b_in == kFusedFlushBlocks - 1;
+                const bool late_b = Cfg::LATE_B && b_in == kFusedFlushBlocks - 1;
                 for (int w = 0; w < WPB; ++w) {
                     if (!ptx::mbar_wait(pp_full(ppb), pp_phase) || !ptx::mbar_wait(full_d(slot), (phase >> slot) & 1u)) { failed = true; break; }
                     ptx::tc_fence_after_sync();
@@ -686,7 +691,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                     if (!SPMM && w == 1 && !late_b && b + 1 < nblk) skip_b();
                 }
                 if (failed) break;
-                if (late_b || b == nblk - 1) ptx::mma_commit(o_full(ch % NOB));
+                if (b_in == kFusedFlushBlocks - 1 || b == nblk - 1) ptx::mma_commit(o_full(ch % NOB));
                 if (!SPMM && late_b && b + 1 < nblk) skip_b();
             }
         }
