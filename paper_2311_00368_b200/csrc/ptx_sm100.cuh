@@ -65,6 +65,16 @@ __device__ __forceinline__ void red_or_shared(uint32_t addr, unsigned m)
     asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(m) : "memory");
 }
 
+// The same where `on` holds; the address need not be valid where it does not.
+__device__ __forceinline__ void red_or_shared_if(uint32_t addr, unsigned m, bool on)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.u32 p, %2, 0;\n\t"
+        "@p red.shared.or.b32 [%0], %1;\n\t}"
+        ::"r"(addr), "r"(m), "r"((unsigned)on) : "memory");
+}
+
 // Four fp32 additions to global memory in one reduction (no return value); 16-byte aligned address.
 __device__ __forceinline__ void red_add_v4(float *addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
 {
