@@ -594,7 +594,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         // eight attention problems 233 -> 211 us, bfloat16 operands (with a ring of eight chunks, not three) 186 -> 165 us,
         // power-law 8192 x 8192 x 128 at 30% 189 -> 181 us.
         if (ptx::elect_one()) {
-            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, 16, 1024, ptx::kLayoutSw128) >> 32);
+            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, 16, 1024, ptx::kLayoutSw128) >> 32), desc0 = (uint32_t)ptx::smem_desc(ring, 16, 1024, ptx::kLayoutSw128);
+            const uint32_t a_desc0 = (uint32_t)ptx::smem_desc(alo_smem, 16, 1024, ptx::kLayoutSw128);
             constexpr uint32_t idesc1 = ptx::idesc_tf32(kFusedRows, kFusedBlk, false, false);
             int slot = 0;
             uint32_t phase = 0;   // per slot: parity of its next B chunk
@@ -618,8 +619,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 const uint32_t pacc = tmem + Cfg::COL_P + pb * kFusedBlk;
                 for (int i = 0; i < NCH_B; ++i) {
                     if (!ptx::mbar_wait(full(slot), (phase >> slot) & 1u)) { failed = true; break; }
-                    const uint32_t b_hi = (uint32_t)ptx::smem_desc(ring + slot * CHUNK, 16, 1024, ptx::kLayoutSw128), b_lo = b_hi + (CHUNK / 2 >> 4);
-                    const uint32_t a_lo = (uint32_t)ptx::smem_desc(alo_smem + i * (kFusedRows * 128), 16, 1024, ptx::kLayoutSw128);
+                    const uint32_t b_hi = desc0 + slot * (CHUNK >> 4), b_lo = b_hi + (CHUNK / 2 >> 4);
+                    const uint32_t a_lo = a_desc0 + i * (kFusedRows * 128 >> 4);
                     const uint32_t acol = tmem + Cfg::COL_AHI + i * 32;
 #pragma unroll
                     for (int k8 = 0; k8 < 4; ++k8) {
@@ -639,13 +640,13 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
     } else if (FUSED && warp == Cfg::G2_WARP) {
         // ---------------- GEMM2 issuer: O += P'_window * D_window ----------------
         if (ptx::elect_one()) {
-            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, kFusedW * 128, 512, ptx::kLayoutSw128Base32) >> 32);
+            const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, kFusedW * 128, 512, ptx::kLayoutSw128Base32) >> 32), desc0 = (uint32_t)ptx::smem_desc(ring, kFusedW * 128, 512, ptx::kLayoutSw128Base32);
             const uint32_t idesc2 = a.NT == 64 ? ptx::idesc_tf32(kFusedRows, 64, false, true) : ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
             constexpr uint32_t idesc2_cat = ptx::idesc_tf32(kFusedRows, kFusedNT, false, true);
-            // 64-column O tiles (N <= 64): a 64-column MMA would leave half of the tensor core's width unused (it takes 46
-            // cycles, not 32), so P'_hi is multiplied by [D_hi | D_lo] in ONE 128-column MMA whose two halves land in
+            // 64-column O tiles (N <= 64): P'_hi is multiplied by [D_hi | D_lo] in ONE 128-column MMA whose two halves land in
             // columns 0-63 and 64-127 of the accumulator, P'_lo by D_hi in a 64-column one: two MMAs per K step instead
-            // of three; the flush adds the two halves.
+            // of three; the flush adds the two halves.  (Three 64-column MMAs would take no longer, but all of them would add into one
+            // accumulator, with truncation: eight attention problems 209 against 211 us, error against float64 3.1e-6 against 2.2e-6.)
             const bool cat = !EXACT && a.NT == 64;
             int slot = NCH_B % RING, ppb = 0;
             uint32_t phase = 0, pp_phase = 0;   // per slot: parity of its next D chunk; parity of the P' buffers' next use
@@ -661,11 +662,11 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                 const uint32_t oacc = tmem + Cfg::COL_O + (ch % NOB) * kFusedNT;
                 const bool late_b = Cfg::LATE_B && b_in == kFusedFlushBlocks - 1;
                 for (int w = 0; w < WPB; ++w) {
-                    if (!ptx::mbar_wait(pp_full(ppb), pp_phase) || !ptx::mbar_wait(full_d(slot), (phase >> slot) & 1u)) { failed = true; break; }
+                    if (!ptx::mbar_wait_both(pp_full(ppb), pp_phase, full_d(slot), (phase >> slot) & 1u)) { failed = true; break; }
                     ptx::tc_fence_after_sync();
                     // D window: MN-major tf32 (32-byte-atom swizzle): column groups 4 KB apart, 4-row K groups 512 B apart,
                     // +1 KB per K step of 8 rows.  (Two copies of the loop: a test inside it costs the issuing thread.)
-                    const uint32_t d_hi = (uint32_t)ptx::smem_desc(ring + slot * CHUNK, kFusedW * 128, 512, ptx::kLayoutSw128Base32), d_lo = d_hi + (CHUNK / 2 >> 4);
+                    const uint32_t d_hi = desc0 + slot * (CHUNK >> 4), d_lo = d_hi + (CHUNK / 2 >> 4);
                     const uint32_t pph = tmem + Cfg::COL_PP + ppb * 64, ppl = pph + 32;
                     const uint32_t first = (b_in | w) != 0;   // 0: this MMA starts a new partial sum
                     if (cat) {
