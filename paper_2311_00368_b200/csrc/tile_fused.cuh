@@ -118,7 +118,6 @@ struct FusedCfg {
     static constexpr bool FUSED = MODE != kModeSddmm;          // has GEMM2 / O
     static constexpr bool SPMM = MODE == kModeSpmm;
     static constexpr int NCH_B = SPMM ? 0 : KDP / 32;          // B chunks per block
-    static constexpr int NCH_D = FUSED ? kFusedBlk / kFusedW : 0;  // D chunks per block
     static constexpr int ALO_BYTES = (FUSED && !SPMM && !EXACT) ? kFusedRows * KDP * 4 : 0;
     // SDDMM runs 28 warps of 72 registers (its processors only copy P, and its helpers work on items of
     // 16 rows, so nobody needs more) with twenty helpers.  FusedMM and SPMM: 20 warps of 96.
@@ -527,7 +526,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
     };
 
     if (warp == kFusedTmaWarp) {
-        // ---------------- TMA producer: per block NCH_B chunks of B rows, then NCH_D chunks of D rows ----------------
+        // ---------------- TMA producer: per block NCH_B chunks of B rows and one chunk of D rows per window ----------------
         if (ptx::elect_one()) {
             if (!SPMM) { ptx::tma_prefetch_desc(&tm_bhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_blo); }
             if (FUSED) { ptx::tma_prefetch_desc(&tm_dhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_dlo); }
