@@ -633,6 +633,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
                     phase ^= 1u << slot;
                     if (++slot == RING) slot = 0;
                 }
+                if (failed) break;   // (a chunk did not arrive: this P is never announced, so nothing computed from it leaves the CTA)
                 ptx::mma_commit(p_full(pb));
             }
         }
