@@ -41,7 +41,7 @@ constexpr int kPatternMagic = 0x62327370;
 // window [32w, 32w+32): bit b set <=> column 32w+b is stored).
 // A row has one mask word per window in shared memory.  First sweep: lane l of a warp reads eight consecutive
 // entries (two 16-byte loads, the next eight in flight meanwhile) and ORs each entry's bit into its window's word.
-// Second sweep: a lane takes four windows; the position of a window is the row start plus the entries of all earlier
+// Second sweep: a lane takes two windows; the position of a window is the row start plus the entries of all earlier
 // windows (a prefix sum over the pop counts).  Every window of every row is written, so the table needs no clearing.
 // The table is only meaningful when the columns of each row are strictly increasing and in range;
 // the first sweep checks exactly that and sets flags[kFlagUnsorted] if not.
@@ -74,6 +74,7 @@ __device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, 
 // entry before the run, `interior` (the same for the whole warp): every lane's run is inside the row.  false: the row is not
 // strictly increasing or out of range (a table with such a row is not used).  Neighbouring lanes are eight entries apart,
 // so that they hardly ever OR into the same word at the same time (consecutive entries mostly share one).
+template <bool SHARED>
 __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev, unsigned p, const TableRow &row, int K, uint32_t words, bool interior)
 {
     auto or_bit = [&](int col) { ptx::red_or_shared(words + 4 * (col >> 5), __funnelshift_l(0u, 1u, col)); };   // 1 << (column within the window)
@@ -86,16 +87,26 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
         for (int i = 0; i < kMasksRun; ++i) or_bit(c[i]);
         return true;
     }
-    // An end of the row: some of the entries are not in it.  Without branches: a row of 820 entries has four chunks, two of them
-    // here.  (This and four windows per lane in the second sweep instead of two: eight FusedMM problems of 4096 x 4096 at 20%, their
-    // table included, 207.9 -> 206.4 us; power-law 8192 x 8192 at 30% 177.4 -> 175.2 us.)
+    // An end of the row: some of the entries are not in it.  Where four warps share a row, without branches (8192 x 8192 at 30%,
+    // Zipf row lengths: 33.2 -> 31.0 us).  With a warp per row that gains nothing at 32768 x 8192 and costs elsewhere, since the eight
+    // predicated steps do not fit into 40 registers (32768 x 512 at 5%: 21.4 -> 22.7 us, 4096 x 30000 at 3%: 14.9 -> 16.5).
     bool bad = false;
+    if constexpr (SHARED) {
 #pragma unroll
-    for (int i = 0; i < kMasksRun; ++i) {
-        const bool in_row = row.has(p + i), in_range = (unsigned)c[i] < (unsigned)K;
-        const bool in_order = p + i == row.beg || c[i] > (i == 0 ? prev : c[i == 0 ? 0 : i - 1]);
-        bad |= in_row & !(in_range & in_order);
-        ptx::red_or_shared_if(words + 4 * (c[i] >> 5), __funnelshift_l(0u, 1u, c[i]), in_row & in_range);
+        for (int i = 0; i < kMasksRun; ++i) {
+            const bool in_row = row.has(p + i), in_range = (unsigned)c[i] < (unsigned)K;
+            const bool in_order = p + i == row.beg || c[i] > (i == 0 ? prev : c[i == 0 ? 0 : i - 1]);
+            bad |= in_row & !(in_range & in_order);
+            ptx::red_or_shared_if(words + 4 * (c[i] >> 5), __funnelshift_l(0u, 1u, c[i]), in_row & in_range);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < kMasksRun; ++i) {
+            if (!row.has(p + i)) continue;
+            const bool in_range = (unsigned)c[i] < (unsigned)K;
+            bad |= !in_range || (p + i != row.beg && c[i] <= (i == 0 ? prev : c[i == 0 ? 0 : i - 1]));
+            if (in_range) or_bit(c[i]);
+        }
     }
     return !bad;
 }
@@ -172,7 +183,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
             int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
             if (lane == 0) prev = !SHARED ? carry : p > tr.beg ? __ldg(col_idx + p - 1) : 0;
             if (!SHARED) carry = __shfl_sync(kFull, c[kMasksRun - 1], 31);
-            bad |= !masks_or_run(c, prev, p, tr, K, mask_smem, p0 >= tr.beg && p0 + kMasksChunk <= tr.end);
+            bad |= !masks_or_run<SHARED>(c, prev, p, tr, K, mask_smem, p0 >= tr.beg && p0 + kMasksChunk <= tr.end);
         }
         if (SHARED) {
             __syncthreads();
@@ -190,7 +201,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
                     masks_load_run(ci, other, p, c);
                     int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
                     if (lane == 0) prev = __ldg(ci + p - 1);
-                    bad |= !masks_or_run(c, prev, p, other, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
+                    bad |= !masks_or_run<SHARED>(c, prev, p, other, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
                 }
                 turn += chunks;
             }
@@ -199,11 +210,14 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
         int run = beg;
         int2 *Trow = T + rowg * Wk;
         const bool pairs = ((rowg * Wk) & 1) == 0;   // the row's records are 16-byte aligned in twos
+        // (Two windows per lane: a warp's stores are contiguous.  With four per lane each store writes half of every 32-byte sector
+        // it touches: 32768 x 2048 at 10% 21.0 -> 22.7 us, 4096 x 60000 at 1% 24.7 -> 27.7, 2500 x 98304 at 1% 18.9 -> 20.6; only
+        // few long runs of windows gained, 32768 x 8192 at 5% 35.0 -> 33.2.)
         if (live)
-            for (int w0 = 0; w0 < Wk; w0 += WARPS * 128) {
-                const int w = w0 + 4 * (SHARED ? (int)threadIdx.x : lane);
-                const uint4 m = w < words ? *reinterpret_cast<const uint4 *>(mask + w) : make_uint4(0u, 0u, 0u, 0u);
-                const int n0 = __popc(m.x), n1 = n0 + __popc(m.y), n2 = n1 + __popc(m.z), cnt = n2 + __popc(m.w);
+            for (int w0 = 0; w0 < Wk; w0 += WARPS * 64) {
+                const int w = w0 + 2 * (SHARED ? (int)threadIdx.x : lane);
+                const uint2 m = w < words ? *reinterpret_cast<const uint2 *>(mask + w) : make_uint2(0u, 0u);
+                const int n0 = __popc(m.x), cnt = n0 + __popc(m.y);
                 int incl = cnt;
 #pragma unroll
                 for (int d = 1; d < 32; d <<= 1) {
@@ -225,14 +239,11 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
                     }
                 }
                 const int pos = run + before + incl - cnt;
-                if (pairs && w + 3 < Wk) {
+                if (pairs && w + 1 < Wk) {
                     *reinterpret_cast<int4 *>(Trow + w) = make_int4(pos, (int)m.x, pos + n0, (int)m.y);
-                    *reinterpret_cast<int4 *>(Trow + w + 2) = make_int4(pos + n1, (int)m.z, pos + n2, (int)m.w);
                 } else {
                     if (w < Wk) Trow[w] = make_int2(pos, (int)m.x);
                     if (w + 1 < Wk) Trow[w + 1] = make_int2(pos + n0, (int)m.y);
-                    if (w + 2 < Wk) Trow[w + 2] = make_int2(pos + n1, (int)m.z);
-                    if (w + 3 < Wk) Trow[w + 3] = make_int2(pos + n2, (int)m.w);
                 }
                 run += all;
                 if (SHARED) __syncthreads();   // warp_total is reused
