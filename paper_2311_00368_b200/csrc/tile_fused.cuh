@@ -154,10 +154,13 @@ struct FusedCfg {
     static constexpr int FLUSH_BUFS = !FUSED ? 0 : ONES || SPMM || EXACT ? 4 : 3;   // per flushing warp: buffers of 32 rows x 16 columns
     static constexpr int FLUSH_BYTES = 4 * FLUSH_BUFS * 2048;
     static constexpr int AUX_BYTES = 1024 /*barriers*/ + kFusedMaxHelpers * 256 /*record tables*/ + SLOTS * SLOT_BYTES + FLUSH_BYTES;
-    // TMA chunks in flight: what the shared memory holds beside the rest.  (ONES with lo halves: three.  With four or five, GEMM1 of
-    // the next block runs ahead of GEMM2 and the eight attention problems take 219 instead of 211 us.)
+    // TMA chunks in flight: what the shared memory holds beside the rest, but three for FusedMM on fp32 operands without stored values
+    // or with 64-wide dot products.  With four, GEMM1 of the next block runs ahead of GEMM2 and takes the tensor core from it (FusedMM on
+    // a prepared table, four -> three: 16384 x 4096, Kd = 64, 15%, N = 64 111.8 -> 108.6 us and N = 128 128.3 -> 121.0; 20000 x 700 at 25%, Kd = 64,
+    // N = 200 91.9 -> 87.8; 8192 x 8192, Kd = N = 64 the same).  With 32-wide ones GEMM1 is half as long and four are better (8192 x 8192,
+    // N = 128, 15%: 116 against 124 us); 128-wide ones leave room for three.
     static constexpr int RING_FIT = (kFusedMaxSmem - ALO_BYTES - 1024 - AUX_BYTES) / CHUNK;
-    static constexpr int RING_MOST = ONES && !EXACT ? 3 : 8;
+    static constexpr int RING_MOST = TWO_ISSUERS && !EXACT && (ONES || KDP == 64) ? 3 : 8;
     static constexpr int RING = RING_FIT < RING_MOST ? RING_FIT : RING_MOST;
     static constexpr int SMEM_BYTES = RING * CHUNK + ALO_BYTES + 1024 + AUX_BYTES;
     // tensor-memory columns
