@@ -200,8 +200,19 @@ b2sp_status pattern_pass(bool prepared, int M, int K, long long nnz, const int *
         if (!allow_dynamic_smem<-1>(reinterpret_cast<const void *>(tile_masks_kernel<true>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
         launch(tile_masks_kernel<true>, rows_all, kMasksSharedWarps * 32, row_bytes);
     } else {
-        if (!allow_dynamic_smem<-2>(reinterpret_cast<const void *>(tile_masks_kernel<false>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
-        launch(tile_masks_kernel<false>, (rows_all + kMasksRows - 1) / kMasksRows, kMasksRows * 32, row_bytes * kMasksRows);
+        // Five blocks per SM do the same work in less time than six, unless that takes another wave: long rows then take six (inputs not in
+        // L2, five against six: 24576 x 4096 rows of 820 entries, five waves against four, 35.2 against 33.6 us; 12288 x 8192, rows of
+        // 2000, three against two, 38.2 against 36.6; 32768 x 4096, rows of 820, six against five, 44.0 against 42.9).  With rows of 500
+        // entries the two are equal (12288 x 4096: 16.4), with shorter ones five are the faster (32768 x 4096, 300: 28.8 against 30.8).
+        const long long blocks = (rows_all + kMasksRows - 1) / kMasksRows;
+        auto waves = [&](bool six) { const int wave = kSMs * masks_blocks_per_sm(six); return (blocks + wave - 1) / wave; };
+        if (nnz / M > 600 && waves(true) < waves(false)) {
+            if (!allow_dynamic_smem<-2>(reinterpret_cast<const void *>(tile_masks_kernel<false, true>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
+            launch(tile_masks_kernel<false, true>, blocks, kMasksRows * 32, row_bytes * kMasksRows);
+        } else {
+            if (!allow_dynamic_smem<-3>(reinterpret_cast<const void *>(tile_masks_kernel<false, false>), kMasksMaxSmem)) return B2SP_ERR_CUDA;
+            launch(tile_masks_kernel<false, false>, blocks, kMasksRows * 32, row_bytes * kMasksRows);
+        }
     }
     *launches += 1;
     return cudaGetLastError() == cudaSuccess ? B2SP_OK : B2SP_ERR_CUDA;

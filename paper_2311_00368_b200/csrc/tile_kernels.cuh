@@ -74,7 +74,7 @@ __device__ __forceinline__ void masks_load_run(const int *__restrict__ col_idx, 
 // entry before the run, `interior` (the same for the whole warp): every lane's run is inside the row.  false: the row is not
 // strictly increasing or out of range (a table with such a row is not used).  Neighbouring lanes are eight entries apart,
 // so that they hardly ever OR into the same word at the same time (consecutive entries mostly share one).
-template <bool SHARED>
+template <bool BRANCH_FREE>
 __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev, unsigned p, const TableRow &row, int K, uint32_t words, bool interior)
 {
     auto or_bit = [&](int col) { ptx::red_or_shared(words + 4 * (col >> 5), __funnelshift_l(0u, 1u, col)); };   // 1 << (column within the window)
@@ -87,11 +87,9 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
         for (int i = 0; i < kMasksRun; ++i) or_bit(c[i]);
         return true;
     }
-    // An end of the row: some of the entries are not in it.  Where four warps share a row, without branches (8192 x 8192 at 30%,
-    // Zipf row lengths: 33.2 -> 31.0 us).  With a warp per row that gains nothing at 32768 x 8192 and costs elsewhere, since the eight
-    // predicated steps do not fit into 40 registers (32768 x 512 at 5%: 21.4 -> 22.7 us, 4096 x 30000 at 3%: 14.9 -> 16.5).
+    // An end of the row: some of the entries are not in it.  (What the two ways cost: at tile_masks_kernel.)
     bool bad = false;
-    if constexpr (SHARED) {
+    if constexpr (BRANCH_FREE) {
 #pragma unroll
         for (int i = 0; i < kMasksRun; ++i) {
             const bool in_row = row.has(p + i), in_range = (unsigned)c[i] < (unsigned)K;
@@ -111,6 +109,9 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
     return !bad;
 }
 
+// Blocks of the form with a warp per row that share an SM.
+constexpr int masks_blocks_per_sm(bool six) { return (six ? 48 : 40) / kMasksRows; }
+
 // A batch of `sig.batch` patterns of the same M and K (row_ptr arrays `sig.rp_stride` elements apart, each
 // starting at 0; col_idx arrays `sig.nz_stride` elements apart) gives one table per pattern, stacked:
 // T[(b*M + r)*Wk + w], positions relative to the pattern's own col_idx array.
@@ -125,8 +126,14 @@ __device__ __forceinline__ bool masks_or_run(const int (&c)[kMasksRun], int prev
 // branches per entry (one 16-byte load per lane and step): 32768 x 8192 at 20% 88 -> 62 us, eight patterns of 4096 x 4096
 // at 20% 61 -> 41 us (those do not begin on 16-byte boundaries), 16384 x 512 at 20% 18 -> 13.5 us, power-law 8192 x 8192 at
 // 30% (SHARED) 38.6 -> 31 us.
-template <bool SHARED>
-__global__ void __launch_bounds__(SHARED ? kMasksSharedWarps * 32 : kMasksRows * 32, SHARED ? 8 : 48 / kMasksRows)
+//
+// SIX: of the form with a warp per row, six blocks per SM (40 registers) instead of five (48).  The ends of rows are handled without
+// branches where the registers allow it, and a row of 410 entries has two chunks, both of them ends.  Five blocks and no branches
+// against six with branches, inputs in L2: 4096 x 4096 at 10% 8.5 against 9.6 us, 8192 x 8192 at 20% 18.6 against 20.4, 16384 x 4096 at 20% 20.7
+// against 22.6, 32768 x 512 at 20% 20.7 against 21.8; power-law 8192 x 8192 at 30% (SHARED) 31.0 against 33.0.  Six blocks without branches
+// spill: 32768 x 512 at 5% 22.7, 4096 x 30000 at 3% 16.5 against 14.7.
+template <bool SHARED, bool SIX = false>
+__global__ void __launch_bounds__(SHARED ? kMasksSharedWarps * 32 : kMasksRows * 32, SHARED ? 8 : masks_blocks_per_sm(SIX))
 tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ row_ptr0,
                   const int *__restrict__ col_idx0, int2 *__restrict__ T, int *__restrict__ flags,
                   PatternSignature sig, PatternSignature *__restrict__ sig_out)
@@ -137,6 +144,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
     ptx::launch_dependents();
     if (blockIdx.x == 0 && threadIdx.x == 0) *sig_out = sig;   // what the table is built from
     constexpr unsigned kFull = 0xffffffffu;
+    constexpr bool BRANCH_FREE = !SIX;
     constexpr int WARPS = SHARED ? kMasksSharedWarps : 1;       // warps of a row
     constexpr int ROWS = SHARED ? 1 : kMasksRows;               // rows of the block at a time
     __shared__ int warp_total[WARPS];
@@ -183,7 +191,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
             int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
             if (lane == 0) prev = !SHARED ? carry : p > tr.beg ? __ldg(col_idx + p - 1) : 0;
             if (!SHARED) carry = __shfl_sync(kFull, c[kMasksRun - 1], 31);
-            bad |= !masks_or_run<SHARED>(c, prev, p, tr, K, mask_smem, p0 >= tr.beg && p0 + kMasksChunk <= tr.end);
+            bad |= !masks_or_run<BRANCH_FREE>(c, prev, p, tr, K, mask_smem, p0 >= tr.beg && p0 + kMasksChunk <= tr.end);
         }
         if (SHARED) {
             __syncthreads();
@@ -201,7 +209,7 @@ tile_masks_kernel(int M, int K, int Wk, long long nnz, const int *__restrict__ r
                     masks_load_run(ci, other, p, c);
                     int prev = __shfl_up_sync(kFull, c[kMasksRun - 1], 1);
                     if (lane == 0) prev = __ldg(ci + p - 1);
-                    bad |= !masks_or_run<SHARED>(c, prev, p, other, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
+                    bad |= !masks_or_run<BRANCH_FREE>(c, prev, p, other, K, ptx::smem_u32(mask_rows + r * words), pc + kMasksChunk <= q.w);
                 }
                 turn += chunks;
             }

@@ -148,3 +148,37 @@ def test_batched_tables(b, batch, M, K, long):
     for i, (r, c) in enumerate(probs):
         want_mask, want_pos = expected(r, c, K)
         assert np.array_equal(mask[i], want_mask) and np.array_equal(pos[i], want_pos)
+
+
+@pytest.mark.parametrize("M,length,long", [
+    (5920, 640, 0),      # 740 blocks of eight rows: one wave with five blocks per SM
+    (5921, 640, 2900),   # two waves with five, one with six: six
+    (7104, 601, 2305),   # the last number of rows for which that holds; just above the length from which it counts
+    (7105, 640, 0),      # two waves either way
+    (6001, 600, 2900),   # rows not long enough
+])
+def test_table_entries_on_either_side_of_the_wave_rule(b, M, length, long):
+    """A warp per row with five or six blocks on an SM (which differ in how the ends of rows are handled): the table, and a column
+    out of order in the first and in the last chunk of a row."""
+    K = 2999
+    rng = np.random.default_rng(M + length)
+    lens = [length + (i % 3) - 1 for i in range(M)]
+    if long:   # a row that is finished by its whole block; the average stays
+        lens[4000] += long - length
+        for i in range(1000):
+            lens[i] -= (long - length + 999 - i) // 1000
+    assert sum(lens) // M == length or sum(lens) // M == length - 1
+    rp, ci = make_rows(rng, lens, K)
+    drp, dci = device(rp, ci, 2)
+    ws = torch.zeros(1 << 25, dtype=torch.uint8, device="cuda")
+    b.prepare_pattern(drp, dci, K, ws)
+    mask, pos = table_of(b, ws, M, K)
+    want_mask, want_pos = expected(rp, ci, K)
+    assert flag_of(b, ws) == 0
+    assert np.array_equal(mask[0], want_mask) and np.array_equal(pos[0], want_pos)
+    for row, entry in ((4321, 1), (4321, int(lens[4321]) - 1), (M - 1, int(lens[M - 1]) - 1), (4000, int(lens[4000]) - 1)):
+        bad, p = ci.copy(), int(rp[row]) + entry
+        bad[p - 1], bad[p] = ci[p], ci[p - 1]
+        drp, dci = device(rp, bad, 2)
+        b.prepare_pattern(drp, dci, K, ws)
+        assert flag_of(b, ws) == 1, (row, entry)
