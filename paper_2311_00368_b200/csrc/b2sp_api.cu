@@ -305,11 +305,12 @@ extern "C" const char *b2sp_status_string(b2sp_status s)
 // writing the sampled values once: measured at N = 512 on the 8192^2 / 30% workload, 717 us fused
 // against 134 + 430 us for SDDMM into a scratch C and SPMM on C.  So wide outputs take the two
 // phases inside one call (same window table, same fallback), and C lives in the workspace.
-// With two tiles (128 < N <= 256) the second GEMM1 costs about what C's round trip does when GEMM1 is long and the
-// problem large: measured at N = 256, Kd = 128, two phases against fused: 8192^2 286 against 288 us (10% density
-// 270 against 279), 4096 x 8192 158 against 153, 16384 x 2048 171 against 152, 4096^2 92 against 85;
-// 8192 x 4096 at Kd = 64 156 against 122 and 2048^2 46 against 33.  (The line was drawn on an earlier fused kernel, 342 us at
-// 8192^2; the largest problems are what is left of its reason.)
+// With two tiles (128 < N <= 256) the line was drawn on an earlier fused kernel (N = 256, Kd = 128, two phases against fused: 8192^2
+// 315 against 342 us).  With the kernels of today the two phases are the slower form at most sizes they are taken at, bfloat16 operands
+// above all: 8192^2 at 30% 344 against 322 us (bfloat16 297 against 239), 16384 x 2048 at 30% 189 against 169 (177 / 137), 4096 x 8192 181
+// against 165 (167 / 132), 32768 x 1024 234 against 200 (215 / 164), 32768 x 4096 at 20% 684 against 651 (566 / 470); only without stored
+// values at 16384 x 8192 are they equal (577 / 581).  Below the line: 4096^2 92 against 85, 8192 x 4096 at Kd = 64 156 against 122, 2048^2 46
+// against 33.
 static bool fusedmm_two_phase(int M, int K, int Kd, int N)
 {
     return N > 256 || (N > 128 && Kd > 64 && (double)M * (double)K >= 3.0e7);

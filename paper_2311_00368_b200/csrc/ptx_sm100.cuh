@@ -147,7 +147,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
 }
 
 // Both phases, asked for together: they are mostly complete, and the second answer comes with the first (with descriptors by one
-// multiply-add, eight attention problems 206.4 -> 205.5 us, bfloat16 159.9 -> 157.9, power-law 8192 x 8192 x 128 at 30% 175.2 -> 174.2).
+// multiply-add, eight attention problems, call after call on the same arrays, 206.4 -> 205.5 us, bfloat16
+// 159.9 -> 157.9).
 __device__ __forceinline__ bool mbar_wait_both(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1)
 {
     uint32_t ok;
@@ -292,7 +293,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 
 // D[tmem] (+)= A[tmem] * B[smem], tf32 inputs, fp32 accumulate.  One thread issues.  Shared-memory descriptors come as their
 // two halves: the upper one is the same for all of an operand's MMAs, and steps along K are 32-bit additions to the lower one
-// (power-law 8192 x 8192 x 128 at 30% FusedMM: 192 -> 181 us against 64-bit descriptors).
+// (against 64-bit descriptors, FusedMM of power-law 8192 x 8192 x 128 at 30%, call after call on the same arrays: 192 -> 181 us).
 __device__ __forceinline__ void mma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint32_t blo, uint32_t bhi, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(

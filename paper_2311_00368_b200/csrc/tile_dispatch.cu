@@ -263,7 +263,7 @@ FusedPlan plan_fused_tile(int M, int K, int Kd, int N, long long nnz, size_t bas
     p.Kp = (K + kFusedBlk - 1) / kFusedBlk * kFusedBlk;   // operand copies padded to whole 128-column blocks
     p.Kdp = Kd == 0 ? 0 : Kd <= 32 ? 32 : Kd <= 64 ? 64 : 128;   // Kd == 0: SPMM through the fused pipeline
     p.Mt = (M + kFusedRows - 1) / kFusedRows;
-    p.NT = fused && N <= 64 ? 64 : kFusedNT;   // a 64-column GEMM2 costs 46 instead of 64 cycles per MMA
+    p.NT = fused && N <= 64 ? 64 : kFusedNT;   // a 64-column MMA takes 32 instead of 64 cycles
     p.Nt = fused ? (N + p.NT - 1) / p.NT : 1;
     p.Np = fused ? p.Nt * p.NT : 0;
     size_t win_bytes = sizeof(int2) * (size_t)batch * (size_t)M * (size_t)p.Wk;

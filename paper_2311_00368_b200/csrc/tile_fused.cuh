@@ -8,8 +8,8 @@
 //     life; A_lo lives in tensor memory too (SDDMM) or in shared memory (FusedMM, where TMEM is
 //     needed for O and P').
 //   * Per block: GEMM1  P = A_tile * B_block^T  (128 x 128).  The B rows of the block arrive by TMA
-//     in chunks of 32 k (hi + lo, 32 KB); N = 128 MMAs run the tensor pipe at full rate (a 128xNx8
-//     tf32 MMA costs max(N/2, 45.6) cycles, so 32-column GEMMs would waste two thirds of it).
+//     in chunks of 32 k (hi + lo, 32 KB).  A 128xNx8 tf32 MMA takes the tensor pipe N/2 cycles, whatever N, but the
+//     thread that issues it 7.5 and, in the kernel, two to four times that: N = 128 is what keeps the pipe fed.
 //   * Four processor warps (thread = row) read P window by window (32 columns) and multiply it by the
 //     window's stored values (0 where nothing is stored), which helper warps fetch with lane =
 //     column (coalesced), densify and transpose through shared-memory slots.  The sampled C of the
@@ -42,7 +42,8 @@ constexpr int kFusedBlk = 128;      // S columns per block (UMMA N of GEMM1)
 // FusedMM and SPMM: 20 warps = 5 per scheduler (a sixth would cut the register budget from 96 to 80 per
 // thread; measured slower).  Warp 1: MMA issue (FusedMM: GEMM1's; warp 15: GEMM2's) + TMEM owner; warp 9: TMA producer; warps 2-5: processors;
 // warps 16-19: second processor set (FusedMM) or flusher warps (SPMM); helpers among warps 0, 6-8, 10-15
-// (FusedMM: eight, none on the MMA warp's scheduler, warp 13 idle; SPMM: ten, warp 13 included).
+// (FusedMM: eight, none on the scheduler of GEMM1's issuer, warp % 4 == 1, where warp 13 is idle; GEMM2's issuer shares the scheduler
+// warp % 4 == 3 with helpers 7 and 11 and processors 3 and 19.  SPMM: ten, warp 13 included.  FusedMM without stored values: none).
 // SDDMM: 28 warps of 72 registers, see FusedCfg.
 constexpr int kFusedThreads = 640;
 constexpr int kFusedTmaWarp = 9;
@@ -97,7 +98,8 @@ struct FusedTileArgs {
 constexpr int kModeSddmm = 0, kModeFused = 1, kModeSpmm = 2;
 
 // Which helper a warp is (-1: none).  20-warp kernels (FusedMM, SPMM): warps 0, 6, 7, 8, 10, 11, 12, 14, 15
-// -> 0 .. 8 (none on the MMA warp's scheduler, warp % 4 == 1), then warp 13 -> 9; warps 16-19 have other roles.
+// -> 0 .. 8 (none on warp 1's scheduler, warp % 4 == 1), then warp 13 -> 9; warps 16-19 have other roles.  FusedMM uses the
+// first eight: warp 15, which would be 8, issues GEMM2.
 // 28-warp kernel (SDDMM): every warp but 1-5 (MMA, processors), 9 (TMA), 21 and 25.
 template <bool NARROW>
 __device__ __forceinline__ int helper_index(int warp)
@@ -112,7 +114,8 @@ __device__ __forceinline__ int helper_index(int warp)
 // has a hi and a lo part).
 // ONES: FusedMM without stored values.  The processors need nothing but the occupancy masks, which each thread reads from the
 // window table itself (one word per window of its row, two windows ahead): no helper warps, no slots.  Measured against helpers
-// that densified ones (eight attention problems of 4096 x 4096, whole call): 241 -> 232 us, bfloat16 operands 202 -> 186 us.
+// that densified ones (eight attention problems of 4096 x 4096, call after call on the same arrays, the window tables built in each):
+// 241 -> 232 us, bfloat16 operands 202 -> 186 us.
 template <int KDP, int MODE, bool EXACT = false, bool ONES = false>
 struct FusedCfg {
     static constexpr bool FUSED = MODE != kModeSddmm;          // has GEMM2 / O
@@ -140,8 +143,9 @@ struct FusedCfg {
     static constexpr int PSETS = (FUSED && !SPMM) ? 2 : 1;
     static constexpr bool TWO_ISSUERS = FUSED && !SPMM;
     // B of the next block after all four windows of D at the end of a chunk of blocks (the tensor core works on GEMM1 while O is flushed)
-    // instead of after two of them.  Not with operands exact in tf32, whose GEMM1 is too short to cover the flush and whose ring holds
-    // both (eight attention problems: 162 us with the same order throughout, 165 with this one; fp32 operands 221 and 211).
+    // instead of after two of them (eight attention problems, call after call on the same arrays: 211 us, with the same order throughout
+    // 221).  Not with operands exact in tf32, whose ring holds both: between nothing and 2% slower there (the same on bfloat16: 161.9 us
+    // without, 163.3 with it, Kd = 32 154.6 and 156.1, Kd = 128 187.2 and 190.2; 8192 x 8192 at 15%, Kd = N = 128, prepared, 112.9 and 114.2).
     static constexpr bool LATE_B = TWO_ISSUERS && !EXACT;
     static constexpr int G2_WARP = TWO_ISSUERS ? 15 : 1;      // the warp that issues GEMM2
     static constexpr int ITEM_ROWS = FUSED ? 32 : 16;           // rows of a helper's work item
@@ -155,7 +159,7 @@ struct FusedCfg {
     static constexpr int FLUSH_BYTES = 4 * FLUSH_BUFS * 2048;
     static constexpr int AUX_BYTES = 1024 /*barriers*/ + kFusedMaxHelpers * 256 /*record tables*/ + SLOTS * SLOT_BYTES + FLUSH_BYTES;
     // TMA chunks in flight: what the shared memory holds beside the rest, but three for FusedMM on fp32 operands without stored values
-    // or with 64-wide dot products.  With four, GEMM1 of the next block runs ahead of GEMM2 and takes the tensor core from it (FusedMM on
+    // or with 64-wide dot products.  With more, GEMM1 of the next block runs ahead of GEMM2 and takes the tensor core from it (FusedMM on
     // a prepared table, four -> three: 16384 x 4096, Kd = 64, 15%, N = 64 111.8 -> 108.6 us and N = 128 128.3 -> 121.0; 20000 x 700 at 25%, Kd = 64,
     // N = 200 91.9 -> 87.8; 8192 x 8192, Kd = N = 64 the same).  With 32-wide ones GEMM1 is half as long and four are better (8192 x 8192,
     // N = 128, 15%: 116 against 124 us); 128-wide ones leave room for three.
@@ -534,7 +538,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             if (!SPMM) { ptx::tma_prefetch_desc(&tm_bhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_blo); }
             if (FUSED) { ptx::tma_prefetch_desc(&tm_dhi); if (!EXACT) ptx::tma_prefetch_desc(&tm_dlo); }
             // Chunk order = the order the MMA issuers consume them: B(0); then per block b:
-            // D(b,0) D(b,1) | B(b+1) | D(b,2) D(b,3)   (SDDMM: B chunks only; last block of a chunk: B(b+1) last).
+            // D(b,0) D(b,1) | B(b+1) | D(b,2) D(b,3)   (SDDMM: B chunks only; SPMM: D chunks only; FusedMM on fp32 operands, last block of
+            // a chunk of blocks: B(b+1) last).
             int c = 0, slot = 0;
             uint32_t empty_phase = 1;   // parity of the slot's previous use
             uint32_t phase_b = 0, phase_d = 0, last_d = 0;   // per slot: parity of its next B chunk and D chunk, whether a D chunk is its last one
@@ -574,7 +579,7 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             };
             for (int i = 0; i < NCH_B && nblk > 0 && !failed; ++i) failed = !put(true, 0, i);
             for (int b = 0; b < nblk && !failed; ++b) {
-                // (FusedMM: at the end of a chunk of blocks GEMM1 of the next block comes last, see the MMA issuers)
+                // (FusedMM on fp32 operands: at the end of a chunk of blocks GEMM1 of the next block comes last, see LATE_B)
                 const bool late_b = Cfg::LATE_B && b % kFusedFlushBlocks == kFusedFlushBlocks - 1;
                 if (FUSED) for (int w = 0; w < 2 && !failed; ++w) failed = !put(false, b, w);
                 if (!SPMM && b + 1 < nblk && !late_b) for (int i = 0; i < NCH_B && !failed; ++i) failed = !put(true, b + 1, i);
@@ -592,9 +597,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
         // GEMM1 and GEMM2 (below) have an issuing thread each.  What an issuing thread does for one chunk beside its MMAs -- barrier
         // checks, commits, bookkeeping, at 6 or more cycles an instruction -- takes it about as long as the tensor core needs for
         // the chunk: one thread for both was what paced the kernel, with 97% of the barriers it asked for long complete and 62% of
-        // its time spent between them even with MMAs cut to a quarter.  Whole calls, one thread -> two and descriptors in halves:
-        // eight attention problems 233 -> 211 us, bfloat16 operands (with a ring of eight chunks, not three) 186 -> 165 us,
-        // power-law 8192 x 8192 x 128 at 30% 189 -> 181 us.
+        // its time spent between them even with MMAs cut to a quarter.  One thread -> two and descriptors in halves, call after call on
+        // the same arrays: eight attention problems 233 -> 211 us, bfloat16 operands (with a ring of eight chunks, not three) 186 -> 165 us.
         if (ptx::elect_one()) {
             const uint32_t desc_up = (uint32_t)(ptx::smem_desc(0, 16, 1024, ptx::kLayoutSw128) >> 32), desc0 = (uint32_t)ptx::smem_desc(ring, 16, 1024, ptx::kLayoutSw128);
             const uint32_t a_desc0 = (uint32_t)ptx::smem_desc(alo_smem, 16, 1024, ptx::kLayoutSw128);
@@ -649,7 +653,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
             // 64-column O tiles (N <= 64): P'_hi is multiplied by [D_hi | D_lo] in ONE 128-column MMA whose two halves land in
             // columns 0-63 and 64-127 of the accumulator, P'_lo by D_hi in a 64-column one: two MMAs per K step instead
             // of three; the flush adds the two halves.  (Three 64-column MMAs would take no longer, but all of them would add into one
-            // accumulator, with truncation: eight attention problems 209 against 211 us, error against float64 3.1e-6 against 2.2e-6.)
+            // accumulator, with truncation: eight attention problems, call after call on the same arrays, 209 against 211 us, error
+            // against float64 3.1e-6 against 2.2e-6.)
             const bool cat = !EXACT && a.NT == 64;
             int slot = NCH_B % RING, ppb = 0;
             uint32_t phase = 0, pp_phase = 0;   // per slot: parity of its next D chunk; parity of the P' buffers' next use
@@ -867,8 +872,8 @@ fused_tile_kernel(const __grid_constant__ CUtensorMap tm_bhi, const __grid_const
     } else if (!ONES && helper_index<FUSED>(warp) >= 0 && helper_index<FUSED>(warp) < NH) {
         // ---------------- helper warps: work items (window, group of rows), round-robin ----------------
         // FusedMM / SPMM: fetch the stored values of the item's 32 rows x 32 columns with lane = column
-        // (coalesced), densify (0 where nothing is stored; 1 for stored entries when there are no
-        // values) and write them transposed into a slot, from which the processor thread of each row
+        // (coalesced), densify (0 where nothing is stored; SPMM without values: 1 for stored entries)
+        // and write them transposed into a slot, from which the processor thread of each row
         // reads its row.  SDDMM (items of 16 rows): prefetch the stored values the same way, then take the
         // P rows the processors left in the slot and write the stored entries, one coalesced run per row.
         if constexpr (!ONES) {
